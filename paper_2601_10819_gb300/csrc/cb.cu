@@ -344,7 +344,12 @@ __device__ __forceinline__ void cb_load8(const __half* p, float* v) {
 template <typename WT>
 __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
     CbHeader* hdr = reinterpret_cast<CbHeader*>(a.ws);
-    if (!hdr->ok) return;
+    // Read once for the whole block: another block of this grid may clear the flag meanwhile (an overfull cell), and
+    // a block that lost some of its warps here would go on with its shared counters unset.
+    __shared__ int s_ok;
+    if (threadIdx.x == 0) s_ok = *reinterpret_cast<volatile int*>(&hdr->ok);
+    __syncthreads();
+    if (!s_ok) return;
     const CbMap* maps = reinterpret_cast<const CbMap*>(a.ws + a.L.maps);
     const long long nbm = (long long)a.B * a.nmaps;
     if ((long long)blockIdx.x >= nbm) {
