@@ -34,7 +34,10 @@ constexpr int kCbWarps = kCbThreads / 32;
 constexpr int kCbMaxMaps = 4096;     // maps the single-block plan kernel can sort
 constexpr int kCbHeavyPerRow = 32;   // expected contributions per row from which a warp sweeps a column
 constexpr unsigned short kNoCell = 0xffffu;
-constexpr int kCbMaxBin = 256;       // points one cell may hold (more: the corner-slot path takes over)
+constexpr int kCbMaxBin = 256;       // points of a cell that a warp sorts in registers
+// Cells of a map whose fuller cells are put in order by reading all points again (a larger map with such a cell hands
+// the gradient to the corner-slot path).  A 68x120 map, the finest of the 1080p set, has 8349.
+constexpr int kCbRescanCells = 9472;
 constexpr int kCbMaxRows = 1024;     // image rows of a map the reduce's band planner holds
 constexpr int kCbDirect = 1 << 30;   // band-end flag: the band is read in place, not staged
 
@@ -293,9 +296,10 @@ __global__ void __launch_bounds__(kCbThreads) cb_plan_kernel(const CbArgs a) {
 // Binning: one block per (batch element, map).  The camera's A * P points get their cells (0xffff when out of
 // view) and are counted per cell with shared-memory atomics; the counts' prefix sums are the map's cell
 // pointers; the points are placed into their cells (shared-memory atomics again) and every cell's points are
-// sorted by point index (one thread per cell of up to 16 points, a warp per fuller cell), which makes the
-// order inside a cell the point order whatever the atomics did.  A cell of more than kCbMaxBin points clears
-// the plan's flag, which hands the whole feature gradient to the corner-slot path.  Then, in record order, each
+// sorted by point index (one thread per cell of up to 16 points, a warp per fuller cell, which sorts up to
+// kCbMaxBin points and reads fuller cells off the points again), which makes the
+// order inside a cell the point order whatever the atomics did.  A cell of more than kCbMaxBin points in a map of
+// more than kCbRescanCells cells clears the plan's flag, which hands the whole feature gradient to the corner-slot path.  Then, in record order, each
 // in-view point gets its anchor's offset a * C/G in grad_out's staged copy and, per group g, the weights of its
 // four corners w_g * (x factor * y factor), in the products every other kernel forms.  Blocks past the maps
 // clear the uncovered rows.
@@ -324,6 +328,23 @@ __device__ __forceinline__ void cb_sort_warp(unsigned short* seg, int n, int lan
     for (int e = 0; e < E; ++e) {
         const int i = lane * E + e;
         if (i < n) seg[i] = (unsigned short)v[e];
+    }
+}
+
+// The points of cell c in point order, read off the cell numbers of all ap points by one warp.  Keypoints projected
+// from boxes crowd into few cells: on 20 cameras of 900 anchors x 13 keypoints (1080p maps) the 17x30 maps have cells of
+// up to 331 points, and handing such a call to the corner-slot path cost 2.9 ms; ap / 32 steps of a warp cost
+// microseconds, and a map of ap points has at most ap / 256 such cells.
+__device__ __forceinline__ void cb_rescan(unsigned short* seg, const unsigned short* cell, int ap, unsigned short c,
+                                          int lane) {
+    const unsigned lt = (1u << lane) - 1u;
+    int n = 0;
+    for (int i0 = 0; i0 < ap; i0 += 32) {
+        const int i = i0 + lane;
+        const bool in = i < ap && cell[i] == c;
+        const unsigned bal = __ballot_sync(0xffffffffu, in);
+        if (in) seg[n + __popc(bal & lt)] = (unsigned short)i;
+        n += __popc(bal);
     }
 }
 
@@ -505,7 +526,7 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
             if (n <= 1) continue;
             if (n <= 4) cb_sort_small<4>(idx + e0, n);
             else if (n <= 16) cb_sort_small<16>(idx + e0, n);
-            else if (n <= kCbMaxBin) lng[atomicAdd(&s_nlong, 1)] = (uint32_t)c;
+            else if (n <= kCbMaxBin || ncell <= kCbRescanCells) lng[atomicAdd(&s_nlong, 1)] = (uint32_t)c;
             else s_abort = 1;
         }
     }
@@ -520,7 +541,8 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
         if (n <= 32) cb_sort_warp<1>(idx + e0, n, lane);
         else if (n <= 64) cb_sort_warp<2>(idx + e0, n, lane);
         else if (n <= 128) cb_sort_warp<4>(idx + e0, n, lane);
-        else cb_sort_warp<8>(idx + e0, n, lane);
+        else if (n <= kCbMaxBin) cb_sort_warp<8>(idx + e0, n, lane);
+        else cb_rescan(idx + e0, cell, ap, (unsigned short)c, lane);
     }
     __syncthreads();
     // records in record order: anchor offsets and the corner coefficients of each group, two at a time
