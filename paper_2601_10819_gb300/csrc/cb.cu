@@ -32,7 +32,8 @@ namespace msda {
 constexpr int kCbThreads = 1024;     // threads of the bin and reduce blocks
 constexpr int kCbWarps = kCbThreads / 32;
 constexpr int kCbMaxMaps = 4096;     // maps the single-block plan kernel can sort
-constexpr int kCbHeavyPerRow = 32;   // expected contributions per row from which a warp sweeps a column
+constexpr int kCbDensePerRow = 4;    // records per feature row of a map from which its cells are summed one by one
+constexpr int kCbWarpPerCell = 16;   // records per cell of a dense map from which a warp sums a cell, not a lane group
 constexpr unsigned short kNoCell = 0xffffu;
 constexpr int kCbMaxBin = 256;       // points of a cell that a warp sorts in registers
 // Cells of a map whose fuller cells are put in order by reading all points again (a larger map with such a cell hands
@@ -41,12 +42,12 @@ constexpr int kCbRescanCells = 9472;
 constexpr int kCbMaxRows = 1024;     // image rows of a map the reduce's band planner holds
 constexpr int kCbDirect = 1 << 30;   // band-end flag: the band is read in place, not staged
 
+constexpr int kCbDensePtrs = 1024;   // cell pointers of a pass over a dense map (in the planner's arrays, two buffers)
+
 struct CbMap {
     int H, W, start;  // W == 0: the map is invalid and skipped
     int cbase;        // first entry of the map in one batch element's cell-pointer array
-    int nseg;         // row segments per column (columns * segments = sweep tasks)
-    int heavy;        // 1: a warp sweeps a column segment; 0: a lane group does
-    int pad[2];
+    int pad[4];
 };
 
 struct CbHeader {
@@ -120,7 +121,7 @@ struct CbRedSmem {
         cptr = aoff + align16(4 * (size_t)(nb + 8));
         bsize = cptr + align16(4 * (size_t)(nb + 8));
         rp = buf + 2 * bsize;
-        bend = rp + align16(4 * (size_t)(kCbMaxRows + 2));
+        bend = rp + align16(4 * (size_t)(kCbMaxRows + 2));  // the two together also hold a dense map's cell pointers
         total = bend + align16(4 * (size_t)kCbMaxRows);
     }
 };
@@ -219,17 +220,10 @@ __global__ void __launch_bounds__(kCbThreads) cb_plan_kernel(const CbArgs a) {
         if (m < nm) {
             const MapInfo mi = load_map(a.shape, a.start, m, a.sum_hw, a.status);
             CbMap cm;
-            cm.H = mi.H; cm.W = mi.W; cm.start = mi.start; cm.cbase = 0; cm.nseg = 1; cm.heavy = 0;
-            cm.pad[0] = cm.pad[1] = 0;
+            cm.H = mi.H; cm.W = mi.W; cm.start = mi.start; cm.cbase = 0;
+            cm.pad[0] = cm.pad[1] = cm.pad[2] = cm.pad[3] = 0;
             if (mi.W != 0) {
                 const long long ncell = (long long)(mi.H + 1) * (mi.W + 1);
-                const long long hw = (long long)mi.H * mi.W;
-                // a warp per column where rows expect many contributions, else a lane group; columns are cut
-                // into row segments until the block's lane groups (warps) have a task each
-                cm.heavy = (4 * ap >= (long long)kCbHeavyPerRow * hw) ? 1 : 0;
-                const int slots = cm.heavy ? kCbWarps : a.nlg;
-                int nseg = slots / mi.W;
-                cm.nseg = nseg < 1 ? 1 : (nseg > mi.H ? mi.H : nseg);
                 if (ncell >= (long long)kNoCell ||
                     align16(4 * (size_t)(ncell + 1)) + cb_bin_fixed(ap) > (size_t)a.bin_smem ||
                     mi.H > kCbMaxRows || 2 * (mi.W + 1) + 9 > a.nb)
@@ -618,9 +612,8 @@ __global__ void __launch_bounds__(256) cb_loc_kernel(const CbArgs a) {
 // finishes, (cy, j), with weight x * (1 - fy), and once to the row below, (cy+1, j), with weight x * fy (x = fx
 // for the left cell, 1 - fx for the right one).  The row below therefore receives its cell-row cy records
 // before its own, which is the order (i-1, j-1), (i-1, j), (i, j-1), (i, j) for every row (i, j); a segment
-// starting at row i0 first sweeps cell row i0 - 1 for the row below only.  Light maps: a lane group (LG lanes,
-// 4 channels each) sweeps a column; heavy maps: a warp does, its lane groups taking every (32/LG)-th record of
-// a cell pair and adding their partial rows with a fixed butterfly when a row is finished.
+// starting at row i0 first sweeps cell row i0 - 1 for the row below only.  A lane group (LG lanes, 4 channels each)
+// sweeps a column.  Dense maps are summed by cells instead (cb_dense_map).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cb_fma4(float4& acc, float k, const float4& v) {
     acc.x = fmaf(k, v.x, acc.x);
@@ -643,18 +636,18 @@ __device__ __forceinline__ void cb_fma2x2(float4& cur, float4& nxt, float kc, fl
     nxt = make_float4(n0.x, n0.y, n1.x, n1.y);
 }
 
-// One cell row of a column from a staged band: records [e, e2) every `step` (record e is coefficient slot
-// e - ce and anchor-offset slot e - ae of the band); records before e1 are the left cell's (corners 1 and 3
-// reach this column: coefficient .y to the finished row, .w to the row below), the others the right cell's
-// (corners 0 and 2: .x and .z).  ONLY_NEXT: the finished row is not this task's.
+// One cell row of a column from a staged band: records [e, e2) (record e is coefficient slot e - ce and anchor-offset
+// slot e - ae of the band); records before e1 are the left cell's (corners 1 and 3 reach this column: coefficient .y to
+// the finished row, .w to the row below), the others the right cell's (corners 0 and 2: .x and .z).  ONLY_NEXT: the
+// finished row is not this task's.
 template <bool ONLY_NEXT>
 __device__ __forceinline__ void cb_step(const uint32_t* __restrict__ Ao, const float4* __restrict__ Cf,
                                         const float4* __restrict__ sgo, int l, uint32_t e, uint32_t e1, uint32_t e2,
-                                        uint32_t ae, uint32_t ce, int step, float4& cur, float4& nxt) {
-    for (; e + step < e2; e += 2 * step) {
-        const uint32_t o0 = Ao[e - ae], o1 = Ao[e + step - ae];
-        const float4 k0 = Cf[e - ce], k1 = Cf[e + step - ce];
-        const bool l0 = e < e1, l1 = e + step < e1;
+                                        uint32_t ae, uint32_t ce, float4& cur, float4& nxt) {
+    for (; e + 1 < e2; e += 2) {
+        const uint32_t o0 = Ao[e - ae], o1 = Ao[e + 1 - ae];
+        const float4 k0 = Cf[e - ce], k1 = Cf[e + 1 - ce];
+        const bool l0 = e < e1, l1 = e + 1 < e1;
         const float4 v0 = sgo[(o0 >> 2) + l];
         const float4 v1 = sgo[(o1 >> 2) + l];
         if (ONLY_NEXT) {
@@ -680,7 +673,7 @@ __device__ __forceinline__ void cb_step(const uint32_t* __restrict__ Ao, const f
 // Band copies of one map: band k covers image rows [i0, i1), so cell rows i0 - 1 .. i1 - 1: their records
 // [rp[i0], rp[i1 + 1]) (coefficients of group g and anchor offsets) and their cell pointers, the pointer and
 // offset ranges rounded out to 16 bytes.  Issued by one thread; completes on `bar`.  A band whose end carries
-// kCbDirect holds rows of which even one exceeds a buffer (cells of hundreds of points in a coarse map): the
+// kCbDirect holds rows of which even one exceeds a buffer (crowded cells): the
 // sweep reads its records and cell pointers from the workspace itself, and its barrier phase completes with a
 // plain arrival, so the buffers' phases stay in step.
 struct CbBand {
@@ -718,14 +711,10 @@ __device__ __forceinline__ CbBand cb_issue_band(const CbArgs& a, unsigned char* 
 // records, anchor offsets and cell pointers taken from the workspace (record e, anchor offset e, cell pointer c
 // at their own indices).  Kept out of line so the staged sweep, which nearly every band takes, is compiled
 // as if it were alone.
-template <int LG>
 __device__ __noinline__ void cb_sweep_in_place(const CbArgs& a, const float4* __restrict__ coef_g,
                                                const float4* __restrict__ sgo, float* gfm, long long pm, int i0,
-                                               int i1, int W, int seg, int ntask, bool heavy, int l, int lgi, int t0,
-                                               int tstep, bool failed) {
-    constexpr int NLGW = 32 / LG;
+                                               int i1, int W, int seg, int ntask, int l, int t0, int tstep, bool failed) {
     const int W1 = W + 1;
-    const int off = heavy ? lgi : 0, step = heavy ? NLGW : 1;
     const uint32_t* Ao = reinterpret_cast<const uint32_t*>(a.ws + a.L.aoff);
     const uint32_t* Cp = reinterpret_cast<const uint32_t*>(a.ws + a.L.cellptr);
     for (int task = t0; task < ntask && !failed; task += tstep) {
@@ -738,25 +727,188 @@ __device__ __noinline__ void cb_sweep_in_place(const CbArgs& a, const float4* __
         for (int cy = r0 - 1; cy < r1; ++cy) {
             const uint32_t q0 = Cp[ci], q1 = Cp[ci + 1], q2 = Cp[ci + 2];
             if (cy < r0) {
-                cb_step<true>(Ao, coef_g, sgo, l, q0 + off, q1, q2, 0u, 0u, step, cur, nxt);
+                cb_step<true>(Ao, coef_g, sgo, l, q0, q1, q2, 0u, 0u, cur, nxt);
             } else {
-                cb_step<false>(Ao, coef_g, sgo, l, q0 + off, q1, q2, 0u, 0u, step, cur, nxt);
-                if (heavy) {
-#pragma unroll
-                    for (int o = LG; o < 32; o <<= 1) {
-                        cur.x += __shfl_xor_sync(0xffffffffu, cur.x, o);
-                        cur.y += __shfl_xor_sync(0xffffffffu, cur.y, o);
-                        cur.z += __shfl_xor_sync(0xffffffffu, cur.z, o);
-                        cur.w += __shfl_xor_sync(0xffffffffu, cur.w, o);
-                    }
-                }
-                if (!heavy || lgi == 0) *reinterpret_cast<float4*>(gfm + ((long long)cy * W + j) * a.C) = cur;
+                cb_step<false>(Ao, coef_g, sgo, l, q0, q1, q2, 0u, 0u, cur, nxt);
+                *reinterpret_cast<float4*>(gfm + ((long long)cy * W + j) * a.C) = cur;
             }
             cur = nxt;
             nxt = make_float4(0.f, 0.f, 0.f, 0.f);
             ci += W1;
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// Dense maps (several records per cell and more: the coarse scales, or keypoints that crowd): whole cells are summed
+// for all four corners at once, every record read once, straight from the workspace, four ahead.  Either a lane group
+// takes a cell, or, with many records per cell (by_warp), the lane groups of a warp share one and then hand the four
+// sums out among themselves; warps take cells from a counter.  The sums are left in shared memory, in the band buffers;
+// when the cells of as many cell rows as fit are summed, the feature rows between them are the sum of four corner sums
+// each, in the order (i-1,j-1), (i-1,j), (i,j-1), (i,j).  Cell row r (cy + 1) lies in slot r % (R + 1), so the last one
+// of a pass stays for the next.  Returns the number of passes, which take the two barriers in turn (each for the cell
+// pointers of a pass, copied while the pass before runs).  Kept out of line so that the column sweeps keep their
+// registers.
+//
+// A column sweep reads a record for each of its two columns, and again for every row segment that a column is cut into
+// to occupy the block.  Measured for one scale alone (64 cameras, 900 anchors, 0.45 M records; a warp sweeping a column
+// of a dense map before): 9x15 maps (44 records per cell) 155 -> 79 us, 17x30 (13 per cell) 127 -> 130 us, whole frame
+// 529 -> 487 us; 16 cameras, batch 4, whole 844 -> 732 us; 20 cameras with projected keypoints, whole 504 -> 394 us.
+// The lines: at 3.3 records per cell (34x60) this form takes 264 us against 143 us for the sweep, whose bands have no
+// passes to start; at 13 a warp per cell takes 150 us against 130 us for a lane group, at 44 79 against 86 us, and
+// where keypoints crowd (projected, 17x30, 21 per cell on average) 88 against 132 us, since a warp evens out its cells.
+// ---------------------------------------------------------------------------
+template <int LG>
+__device__ __noinline__ int cb_dense_map(const CbArgs& a, const float4* __restrict__ coef_g,
+                                         const float4* __restrict__ sgo, float4* scratch, int ncap, float* gfm,
+                                         long long pm, int H, int W, uint32_t* cptr, int* ctr, int* fail, uint64_t* mbar,
+                                         uint32_t ph0, uint32_t ph1, bool by_warp) {
+    constexpr int NLGW = 32 / LG;
+    constexpr int U = 4;
+    const int W1 = W + 1, R = ncap / W1 - 1;  // cell rows of a pass
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lgi = lane / LG, l = lane % LG;
+    const uint32_t* Ao = reinterpret_cast<const uint32_t*>(a.ws + a.L.aoff);
+    // the cell pointers of a pass, rounded out to 16 bytes, in buffer bf of two (by thread 0)
+    auto issue = [&](int r, int bf) {
+        const long long c0 = (pm + (long long)r * W1) & ~3ll, c1 = (pm + (long long)min(r + R, H + 1) * W1 + 4) & ~3ll;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the threads' reads of this buffer come first
+        mbar_arrive_expect_tx(&mbar[bf], (uint32_t)(c1 - c0) * 4u);
+        bulk_load(cptr + bf * kCbDensePtrs, reinterpret_cast<const uint32_t*>(a.ws + a.L.cellptr) + c0,
+                  (uint32_t)(c1 - c0) * 4u, &mbar[bf]);
+    };
+    if (threadIdx.x == 0) issue(0, 0);
+    int npass = 0;
+    for (int r0 = 0, bf = 0; r0 <= H; r0 += R, bf ^= 1, ++npass) {
+        const int r1 = min(r0 + R, H + 1);
+        if (threadIdx.x == 0) {
+            if (r1 <= H) issue(r1, bf ^ 1);
+            *ctr = kCbWarps;
+            const uint32_t par = bf ? ph1 : ph0;
+            if (!mbar_wait_first(&mbar[bf], par)) {
+                *fail = 1;
+                raise_status(a.status, MSDA_ERR_TIMEOUT);
+                mbar_wait_drain(&mbar[bf], par);  // the copy in flight lands before the buffer is reused
+            }
+        }
+        if (bf) ph1 ^= 1u; else ph0 ^= 1u;
+        __syncthreads();  // pointers and counter are there, and the rows of the pass before are assembled
+        const int ncell = *fail ? 0 : (r1 - r0) * W1;
+        const uint32_t* Cp = cptr + bf * kCbDensePtrs + ((pm + (long long)r0 * W1) & 3);
+        if (!by_warp) {
+            // a lane group per cell: the lane groups of a warp take NLGW consecutive cells
+            for (int c0 = warp * NLGW; c0 < ncell;) {
+                const int c = c0 + lgi;
+                const uint32_t e0 = c < ncell ? Cp[c] : 0u, e1 = c < ncell ? Cp[c + 1] : 0u;
+                float4 s[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) s[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (uint32_t e = e0; e < e1; e += U) {
+                    uint32_t o[U];
+                    float4 k[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const uint32_t eu = min(e + u, e1 - 1);
+                        o[u] = __ldg(Ao + eu);
+                        k[u] = __ldg(coef_g + eu);
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        if (e + u < e1) {
+                            const float4 v = sgo[(o[u] >> 2) + l];
+                            cb_fma2x2(s[0], s[1], k[u].x, k[u].y, v);
+                            cb_fma2x2(s[2], s[3], k[u].z, k[u].w, v);
+                        }
+                    }
+                }
+                if (c < ncell) {
+                    float4* dst = scratch + ((long long)(((r0 + c / W1) % (R + 1)) * W1 + c % W1) * 4) * LG + l;
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) dst[q * LG] = s[q];
+                }
+                if (lane == 0) c0 = atomicAdd(ctr, 1) * NLGW;
+                c0 = __shfl_sync(0xffffffffu, c0, 0);
+            }
+        }
+        for (int c = by_warp ? warp : ncell; c < ncell;) {
+            const uint32_t e0 = Cp[c], e1 = Cp[c + 1];
+            float4 s[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) s[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (uint32_t e = e0 + lgi; e < e1; e += U * NLGW) {
+                uint32_t o[U];
+                float4 k[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const uint32_t eu = min(e + u * NLGW, e1 - 1);
+                    o[u] = __ldg(Ao + eu);
+                    k[u] = __ldg(coef_g + eu);
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (e + u * NLGW < e1) {
+                        const float4 v = sgo[(o[u] >> 2) + l];
+                        cb_fma2x2(s[0], s[1], k[u].x, k[u].y, v);
+                        cb_fma2x2(s[2], s[3], k[u].z, k[u].w, v);
+                    }
+                }
+            }
+            // the lane groups' shares, summed: plain butterflies while more than four lane groups are left, then the
+            // corners are halved between the lanes, so that corner q ends in the lanes of index q among four (two
+            // corners each among two lane groups, all four in one)
+            auto xadd = [](float4& x, const float4& y, int o) {
+                x.x += __shfl_xor_sync(0xffffffffu, y.x, o);
+                x.y += __shfl_xor_sync(0xffffffffu, y.y, o);
+                x.z += __shfl_xor_sync(0xffffffffu, y.z, o);
+                x.w += __shfl_xor_sync(0xffffffffu, y.w, o);
+            };
+            auto pick = [](bool p, const float4& x, const float4& y) {
+                return make_float4(p ? x.x : y.x, p ? x.y : y.y, p ? x.z : y.z, p ? x.w : y.w);
+            };
+#pragma unroll
+            for (int off = LG; off < 8; off <<= 1)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float4 t = s[q];
+                    xadd(s[q], t, off);
+                }
+            float4* dst = scratch + ((long long)(((r0 + c / W1) % (R + 1)) * W1 + c % W1) * 4) * LG + l;
+            if constexpr (LG <= 16) {
+                const bool up = lane & 16;
+                float4 k0 = pick(up, s[2], s[0]), k1 = pick(up, s[3], s[1]);
+                xadd(k0, pick(up, s[0], s[2]), 16);
+                xadd(k1, pick(up, s[1], s[3]), 16);
+                if constexpr (LG == 16) {
+                    dst[2 * lgi * LG] = k0;
+                    dst[(2 * lgi + 1) * LG] = k1;
+                } else {
+                    const bool odd = lane & 8;
+                    float4 k2 = pick(odd, k1, k0);
+                    xadd(k2, pick(odd, k0, k1), 8);
+                    if (LG == 8 || (lane & 7) < LG) dst[(lane >> 3) * LG] = k2;
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) dst[q * LG] = s[q];
+            }
+            if (lane == 0) c = atomicAdd(ctr, 1);
+            c = __shfl_sync(0xffffffffu, c, 0);
+        }
+        __syncthreads();
+        // feature rows whose two cell rows (i and i + 1 in this numbering) are both summed
+        const int i0 = r0 > 0 ? r0 - 1 : 0, nrow = *fail ? 0 : (r1 - 1 - i0) * W;
+        for (int t = warp * NLGW + lgi; t < nrow; t += kCbWarps * NLGW) {
+            const int i = i0 + t / W, j = t % W;
+            const float4* up = scratch + ((long long)((i % (R + 1)) * W1 + j) * 4) * LG + l;
+            const float4* dn = scratch + ((long long)(((i + 1) % (R + 1)) * W1 + j) * 4) * LG + l;
+            const float4 x3 = up[3 * LG], x2 = up[(4 + 2) * LG], x1 = dn[1 * LG], x0 = dn[4 * LG];
+            *reinterpret_cast<float4*>(gfm + ((long long)i * W + j) * a.C) =
+                make_float4(x3.x + x2.x + x1.x + x0.x, x3.y + x2.y + x1.y + x0.y, x3.z + x2.z + x1.z + x0.z,
+                            x3.w + x2.w + x1.w + x0.w);
+        }
+        __syncthreads();
+    }
+    return npass;
 }
 
 template <int LG>
@@ -779,10 +931,10 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
     int* bend = reinterpret_cast<int*>(smem + L.bend);
     __shared__ uint64_t mbar[2];
     __shared__ CbBand s_band[2];
-    __shared__ int s_item[2], s_nb, s_fail;
+    __shared__ int s_item[2], s_nb, s_fail, s_ctr;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int lgi = lane / LG, l = lane % LG;
-    const int lgid = warp * NLGW + lgi;
+    const int l = lane % LG;
+    const int lgid = warp * NLGW + lane / LG;
     const int nlg = kCbWarps * NLGW;
     const int cg4 = a.Cg / 4;
     if (threadIdx.x == 0) {
@@ -811,6 +963,21 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
             if (mp.W != 0) {
                 const int H = mp.H, W = mp.W, W1 = W + 1;
                 const long long pm = (long long)b * a.L.nccap + mp.cbase;  // the map's cell pointers
+                float* gfm = gfb + (long long)mp.start * a.C;
+                // a dense map takes its cells one by one, if the corner sums of two cell rows fit in the band buffers
+                const int ncap = min((int)(2 * L.bsize / (4 * sizeof(float) * (size_t)a.Cg)), kCbDensePtrs - 8);
+                const uint32_t nrec = __ldg(cellptr + pm + (long long)(H + 1) * W1) - __ldg(cellptr + pm);
+                if (nrec >= (uint32_t)kCbDensePerRow * (uint32_t)(H * W) && 2 * W1 <= ncap) {
+                    const int npass = cb_dense_map<LG>(a, coef_g, sgo, reinterpret_cast<float4*>(buf0), ncap, gfm, pm, H, W, rp, &s_ctr,
+                                     &s_fail, mbar, ph0, ph1,
+                                     nrec >= (uint32_t)kCbWarpPerCell * (uint32_t)((H + 1) * W1));
+                    ph0 ^= (uint32_t)((npass + 1) / 2) & 1u;  // the passes took the two barriers in turn
+                    ph1 ^= (uint32_t)(npass / 2) & 1u;
+                    // bulk copies of the next map's bands come after these reads and writes of the buffers
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncthreads();
+                    continue;
+                }
                 // record starts of the cell rows (cell row index r = cy + 1), then the bands
                 for (int r = threadIdx.x; r <= H + 1; r += blockDim.x) rp[r] = __ldg(cellptr + pm + (long long)r * W1);
                 __syncthreads();
@@ -847,8 +1014,6 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
                         s_band[k] = cb_issue_band(a, buf0 + k * L.bsize, L, rp, k ? bend[k - 1] & ~kCbDirect : 0,
                                                   bend[k], pm, W1, coef_g, &mbar[k]);
                 }
-                float* gfm = gfb + (long long)mp.start * a.C;
-                const bool heavy = mp.heavy != 0;
                 for (int k = 0; k < nb; ++k) {
                     const int bf = k & 1;
                     const uint32_t par = bf ? ph1 : ph0;
@@ -864,22 +1029,18 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
                     const CbBand bd = s_band[bf];
                     const unsigned char* bb = buf0 + bf * L.bsize;
                     const int R = i1 - i0;
-                    const int slots = heavy ? kCbWarps : nlg;
-                    int S = slots / W;
+                    int S = nlg / W;
                     S = S < 1 ? 1 : (S > R ? R : S);
                     const int seg = (R + S - 1) / S;
                     const int ntask = W * S;
-                    const int t0 = heavy ? warp : lgid, tstep = heavy ? kCbWarps : nlg;
-                    const int off = heavy ? lgi : 0, step = heavy ? NLGW : 1;
                     const bool failed = s_fail != 0;
                     if (direct) {
-                        cb_sweep_in_place<LG>(a, coef_g, sgo, gfm, pm, i0, i1, W, seg, ntask, heavy, l, lgi,
-                                              t0, tstep, failed);
+                        cb_sweep_in_place(a, coef_g, sgo, gfm, pm, i0, i1, W, seg, ntask, l, lgid, nlg, failed);
                     } else {
                         const float4* Cf = reinterpret_cast<const float4*>(bb);
                         const uint32_t* Ao = reinterpret_cast<const uint32_t*>(bb + L.aoff);
                         const uint32_t* Cp = reinterpret_cast<const uint32_t*>(bb + L.cptr);
-                        for (int task = t0; task < ntask && !failed; task += tstep) {
+                        for (int task = lgid; task < ntask && !failed; task += nlg) {
                             const int sg = task / W, j = task - sg * W;
                             const int r0 = i0 + sg * seg, r1 = min(r0 + seg, i1);
                             if (r0 >= r1) continue;
@@ -890,20 +1051,10 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
                             for (int cy = r0 - 1; cy < r1; ++cy) {
                                 const uint32_t q0 = Cp[ci], q1 = Cp[ci + 1], q2 = Cp[ci + 2];
                                 if (cy < r0) {
-                                    cb_step<true>(Ao, Cf, sgo, l, q0 + off, q1, q2, bd.ea0, bd.e0, step, cur, nxt);
+                                    cb_step<true>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, cur, nxt);
                                 } else {
-                                    cb_step<false>(Ao, Cf, sgo, l, q0 + off, q1, q2, bd.ea0, bd.e0, step, cur, nxt);
-                                    if (heavy) {
-#pragma unroll
-                                        for (int o = LG; o < 32; o <<= 1) {
-                                            cur.x += __shfl_xor_sync(0xffffffffu, cur.x, o);
-                                            cur.y += __shfl_xor_sync(0xffffffffu, cur.y, o);
-                                            cur.z += __shfl_xor_sync(0xffffffffu, cur.z, o);
-                                            cur.w += __shfl_xor_sync(0xffffffffu, cur.w, o);
-                                        }
-                                    }
-                                    if (!heavy || lgi == 0)
-                                        *reinterpret_cast<float4*>(gfm + ((long long)cy * W + j) * a.C) = cur;
+                                    cb_step<false>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, cur, nxt);
+                                    *reinterpret_cast<float4*>(gfm + ((long long)cy * W + j) * a.C) = cur;
                                 }
                                 cur = nxt;
                                 nxt = make_float4(0.f, 0.f, 0.f, 0.f);
