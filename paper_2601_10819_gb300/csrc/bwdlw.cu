@@ -1,8 +1,9 @@
-// MSDA backward, location and weight gradients, one block per anchor (sm_103a).
+// MSDA backward, location and weight gradients, one block per anchor and
+// camera group (sm_103a).
 //
 // The deterministic backward takes dloc and dw from this kernel (its feature
-// gradient comes from the sort-and-reduce path of det.cu).  The block lists
-// its anchor's in-view point-scales once (units.cuh) and deals them to teams
+// gradient comes from cb.cu or det.cu).  The block lists its anchor's
+// in-view point-scales once (units.cuh) and deals them to teams
 // of rt lanes, each lane holding its slice of the anchor's grad_out row in
 // registers.  For a point-scale the team dots the four corner rows with
 // grad_out (d_q, per lane over its channels) and forms, with the bilinear
@@ -15,8 +16,16 @@
 // is their sum, scaled by W_s and H_s, in scale order at the end.  A
 // point-scale that is not listed gets dw = 0, a point with no listed scale
 // dloc = 0.  Every sum has a fixed order, so the result is bitwise
-// reproducible.  An anchor whose locations and sums do not fit in shared
-// memory falls back to the per-point kernel of bwd.cu without its scatter.
+// reproducible.  Nothing is summed over cameras, so a block takes only as
+// many cameras as one list chunk covers (16 of 64 with 13 keypoints and 4
+// scales), in the order of batch element, group, anchor: the blocks that run
+// together read the maps of the same few cameras, and there are enough of them that the last wave is
+// short and that few anchors still fill the GPU.  Alone on the GPU, 64
+// cameras of 1080p maps, 4 warps: 900 anchors 695 -> 397 us, 100 anchors
+// 355 -> 80 us (one block per anchor and all its cameras before).  The
+// latency of the corner rows bounds it (3.5 GB from L2, 180 us at the probed
+// gather rate), with three blocks of 8 warps, or six of 4, per SM.  A camera
+// whose locations and sums do not fit in shared memory falls back to the per-point kernel of bwd.cu without its scatter.
 #include "common.cuh"
 #include "internal.h"
 #include "units.cuh"
@@ -34,11 +43,12 @@ struct LocWArgs {
     float* gw;
     int B, sum_hw, C, Ncam, Nscale, A, P, G, Cg;
     int rt;
-    int wide;  // 256-bit corner loads (NV = 2, 32-byte aligned rows)
+    int wide;   // 256-bit corner loads (NV = 2, 32-byte aligned rows)
+    int gcams;  // cameras per block
     int* status;
 };
 
-// Shared memory: map table, camera boxes, locations, per point-scale (du, dv), point-scale list.
+// Shared memory: the group's map table, camera boxes, locations, per point-scale (du, dv), point-scale list.
 struct LocWSmem {
     size_t maps, box, loc, uv, list, total;
     __host__ __device__ LocWSmem(int nmaps, int P, int Ncam, int Nscale, int units) {
@@ -77,24 +87,37 @@ __global__ void __launch_bounds__(256, NV == 2 ? 3 : (NV == 1 ? 4 : 2)) bwd_locw
     constexpr int VEC = Elem<FT>::VEC;
     constexpr int CPL = VEC * NV;
     extern __shared__ __align__(16) unsigned char smem[];
-    const int nmaps = p.Ncam * p.Nscale;
-    const int per_point = p.P * p.Ncam;
+    // blocks by batch element, then camera group, then anchor
+    const unsigned bc = blockIdx.x / (unsigned)p.A, ngroups = gridDim.x / ((unsigned)p.B * (unsigned)p.A);
+    const int b = (int)(bc / ngroups);
+    const long long ba = (long long)b * p.A + (blockIdx.x - bc * (unsigned)p.A);
+    const int k0 = (int)(bc - b * ngroups) * p.gcams, ncam = min(p.gcams, p.Ncam - k0);  // this block's cameras
+    // what the end needs again is not held in registers across the main loop
+    __shared__ long long s_anchor;
+    __shared__ int2 s_slice;
+    if (threadIdx.x == 0) {
+        s_anchor = ba;
+        s_slice = make_int2(k0, ncam);
+    }
+    const int per_point = p.P * ncam;
     const int npts = per_point * p.Nscale;
-    const LocWSmem lay(nmaps, p.P, p.Ncam, p.Nscale, (int)blockDim.x * kUnitsPerThread);
+    const LocWSmem lay(p.gcams * p.Nscale, p.P, p.gcams, p.Nscale, (int)blockDim.x * kUnitsPerThread);
     MapInfo* smap = reinterpret_cast<MapInfo*>(smem + lay.maps);
     float4* sbox = reinterpret_cast<float4*>(smem + lay.box);
     float2* sloc = reinterpret_cast<float2*>(smem + lay.loc);
     float2* suv = reinterpret_cast<float2*>(smem + lay.uv);
     const UnitList ul(smem + lay.list, (int)blockDim.x * kUnitsPerThread);
 
-    const long long ba = blockIdx.x;
-    const int b = (int)(ba / p.A);
-    for (int i = threadIdx.x; i < nmaps; i += blockDim.x) smap[i] = load_map(p.shape, p.start, i, p.sum_hw, p.status);
-    const float2* gl = reinterpret_cast<const float2*>(p.loc) + ba * (long long)per_point;
-    for (int i = threadIdx.x; i < per_point; i += blockDim.x) sloc[i] = __ldg(gl + i);
+    for (int i = threadIdx.x; i < ncam * p.Nscale; i += blockDim.x)
+        smap[i] = load_map(p.shape, p.start, k0 * p.Nscale + i, p.sum_hw, p.status);
+    const float2* gl = reinterpret_cast<const float2*>(p.loc) + ba * (long long)(p.P * p.Ncam) + k0;
+    for (int i = threadIdx.x; i < per_point; i += blockDim.x) {
+        const int pp = i / ncam;
+        sloc[i] = __ldg(gl + (long long)pp * p.Ncam + (i - pp * ncam));
+    }
     for (int i = threadIdx.x; i < npts; i += blockDim.x) suv[i] = make_float2(0.0f, 0.0f);
     __syncthreads();
-    for (int k = threadIdx.x; k < p.Ncam; k += blockDim.x) sbox[k] = camera_box(smap + k * p.Nscale, p.Nscale);
+    for (int k = threadIdx.x; k < ncam; k += blockDim.x) sbox[k] = camera_box(smap + k * p.Nscale, p.Nscale);
     __syncthreads();
 
     const int tpw = 32 / p.rt;
@@ -108,8 +131,10 @@ __global__ void __launch_bounds__(256, NV == 2 ? 3 : (NV == 1 ? 4 : 2)) bwd_locw
     const int g = c0 / p.Cg;
     const int lg = p.Cg / CPL;  // lanes per group
     const FT* fb = reinterpret_cast<const FT*>(p.feat) + (long long)b * p.sum_hw * p.C + c0;
-    const WT* wb = reinterpret_cast<const WT*>(p.w) + ba * (long long)npts * p.G;
-    float* gwb = p.gw + ba * (long long)npts * p.G;
+    // weights and their gradients: point-scale (k0 + k, pp, s) of the anchor is row (pp * Ncam + k) * Nscale + s
+    const long long wrow0 = (ba * p.P * p.Ncam + k0) * p.Nscale;
+    const WT* wb = reinterpret_cast<const WT*>(p.w) + wrow0 * p.G;
+    float* gwb = p.gw + wrow0 * p.G;
     float2 go[CPL / 2];
 #pragma unroll
     for (int j = 0; j < CPL / 4; ++j) {
@@ -120,10 +145,10 @@ __global__ void __launch_bounds__(256, NV == 2 ? 3 : (NV == 1 ? 4 : 2)) bwd_locw
 
     const int chunk = blockDim.x * kUnitsPerThread;
     for (int u0 = 0; u0 < npts; u0 += chunk) {
-        const int G = p.G, Ncam = p.Ncam, Nscale = p.Nscale;
-        const int total = build_unit_list(u0, npts, p.P, p.Ncam, p.Nscale, smap, sbox, sloc, nullptr, ul,
-                                          [&](int pp, int k, int sc) {
-                                              float* d = gwb + ((long long)((pp * Ncam + k) * Nscale + sc)) * G;
+        const int G = p.G;
+        const int total = build_unit_list(u0, npts, p.P, s_slice.y, p.Nscale, p.Ncam, smap, sbox, sloc, nullptr, ul,
+                                          [&](int row) {
+                                              float* d = gwb + (long long)row * G;
                                               if ((G & 3) == 0) {  // 16-byte aligned rows of G values
                                                   for (int gg = 0; gg < G; gg += 4)
                                                       *reinterpret_cast<float4*>(d + gg) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -176,21 +201,23 @@ __global__ void __launch_bounds__(256, NV == 2 ? 3 : (NV == 1 ? 4 : 2)) bwd_locw
             float du = wv * (ay * (d01 - d00) + r.fy * (d11 - d10));
             float dv = wv * (ax * (d10 - d00) + r.fx * (d11 - d01));
             team_sum2_lw(du, dv, tmask, p.rt);
-            if (tl == 0) suv[ps] = make_float2(du, dv);  // scaled by W_s, H_s at the end
+            if (tl == 0) suv[__float_as_int(r.scale)] = make_float2(du, dv);  // scaled by W_s, H_s at the end
         }
         __syncthreads();  // the list is rebuilt for the next chunk; suv is complete after the last one
     }
     // dloc of each point: its scales' terms in scale order
-    float2* glb = reinterpret_cast<float2*>(p.gloc) + ba * (long long)per_point;
-    for (int pt = threadIdx.x; pt < per_point; pt += blockDim.x) {
-        const MapInfo* mrow = smap + (pt % p.Ncam) * p.Nscale;
+    const int ncam1 = s_slice.y;
+    float2* glb = reinterpret_cast<float2*>(p.gloc) + s_anchor * (long long)(p.P * p.Ncam) + s_slice.x;
+    for (int i = threadIdx.x; i < p.P * ncam1; i += blockDim.x) {
+        const int pp = i / ncam1, k = i - pp * ncam1;
+        const MapInfo* mrow = smap + k * p.Nscale;
+        const float2* t = suv + (k * p.P + pp) * p.Nscale;
         float du = 0.0f, dv = 0.0f;
         for (int s = 0; s < p.Nscale; ++s) {
-            const float2 t = suv[pt * p.Nscale + s];
-            du = fmaf((float)mrow[s].W, t.x, du);
-            dv = fmaf((float)mrow[s].H, t.y, dv);
+            du = fmaf((float)mrow[s].W, t[s].x, du);
+            dv = fmaf((float)mrow[s].H, t[s].y, dv);
         }
-        glb[pt] = make_float2(du, dv);
+        glb[(long long)pp * p.Ncam + k] = make_float2(du, dv);
     }
 }
 
@@ -227,7 +254,18 @@ msda_status launch_backward_locw(const Problem& p, const float* grad_out, float*
     if (nblocks > 0x7fffffffLL) return fail(MSDA_ERR_UNSUPPORTED, "msda_backward: B*A too large");
     if ((long long)p.P * p.Ncam * p.Nscale >= (1ll << 26))
         return fail(MSDA_ERR_UNSUPPORTED, "msda_backward: too many point-scales per anchor");
-    const LocWSmem lay(p.Ncam * p.Nscale, p.P, p.Ncam, p.Nscale, warps * 32 * kUnitsPerThread);
+    // Camera groups: one chunk of point-scales each, where a camera does not exceed a chunk, spread evenly (half and
+    // twice as many cameras per block were within 5 % on 64 cameras, 4 warps against 8).
+    const int chunk = warps * 32 * kUnitsPerThread;
+    const long long per_cam = (long long)p.P * p.Nscale;
+    int gcams = p.Ncam > 0 ? p.Ncam : 1, ngroups = 1;
+    if (per_cam > 0 && p.Ncam > 0 && nblocks * p.Ncam <= 0x7fffffffLL) {
+        gcams = per_cam >= chunk ? 1 : (int)(chunk / per_cam);
+        ngroups = (p.Ncam + gcams - 1) / gcams;
+        gcams = (p.Ncam + ngroups - 1) / ngroups;
+        ngroups = (p.Ncam + gcams - 1) / gcams;
+    }
+    const LocWSmem lay(gcams * p.Nscale, p.P, gcams, p.Nscale, chunk);
     if (lay.total > (size_t)dev.max_smem_optin)  // an anchor too large to stage: the per-point kernel
         return launch_backward_loc_w(p, grad_out, nullptr, grad_loc, grad_w, warps, 0, stream);
     st = ensure_smem((const void*)k, lay.total, dev);
@@ -240,7 +278,8 @@ msda_status launch_backward_locw(const Problem& p, const float* grad_out, float*
     const size_t esz = (size_t)dtype_size(p.feat_t);
     a.wide = (p.nv == 2 && ((uintptr_t)p.feat % 32) == 0 && ((size_t)p.C * esz) % 32 == 0 &&
               ((size_t)p.sum_hw * p.C * esz) % 32 == 0) ? 1 : 0;
-    k<<<(unsigned)nblocks, warps * 32, lay.total, stream>>>(a);
+    a.gcams = gcams;
+    k<<<(unsigned)(nblocks * ngroups), warps * 32, lay.total, stream>>>(a);
     return check_launch("msda_backward dloc/dw");
 }
 

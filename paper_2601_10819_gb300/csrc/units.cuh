@@ -25,7 +25,8 @@ struct UnitRec {
     int W;       // map width: rows between y0 and y0 + 1
     float fx, fy;
     int wf;      // (index of the point-scale's weights) << 4 | vx0 | vx1 << 1 | vy0 << 2 | vy1 << 3
-    float scale; // camera factor of the fused occlusion-aware form, else 1
+    float scale; // forward kernels: camera factor of the fused occlusion-aware form, else 1; build_unit_list without
+                 // camera factors: the point-scale's number u (the bits of an int)
 };
 
 // Bytes of the record array, its 2-byte list and the scan scratch for `units` entries.
@@ -72,24 +73,25 @@ struct UnitList {
 };
 
 // Stage A for the chunk starting at u0: returns the number of listed point-scales (the same in every thread).
-// dropped(pp, k, s) is called, by the thread that owns it, for each point-scale of the chunk that is not
-// listed.  Ends with a block barrier, so the list is ready for stage B.
+// A point-scale's weights are row (pp * pitch + k) * Nscale + s of the caller's (pitch: cameras between two keypoints,
+// Ncam unless the caller's cameras are a slice).  dropped(row) is called, by the thread that owns it, for each
+// point-scale of the chunk that is not listed.  Ends with a block barrier, so the list is ready for stage B.
 template <typename Dropped>
-__device__ __forceinline__ int build_unit_list(int u0, int nunits, int P, int Ncam, int Nscale,
+__device__ __forceinline__ int build_unit_list(int u0, int nunits, int P, int Ncam, int Nscale, int pitch,
                                                const MapInfo* __restrict__ smap, const float4* __restrict__ sbox,
                                                const float2* __restrict__ sloc, const float* __restrict__ svn,
                                                const UnitList& ul, Dropped dropped) {
     const int per_cam = P * Nscale;
     const int mine = (int)threadIdx.x * kUnitsPerThread;
     unsigned vmask = 0u;
+    // the thread's point-scales are consecutive: decoded once, then counted on
+    int k = (u0 + mine) / per_cam;
+    int pp = (u0 + mine - k * per_cam) / Nscale;
+    int sc = u0 + mine - k * per_cam - pp * Nscale;
 #pragma unroll
     for (int i = 0; i < kUnitsPerThread; ++i) {
         const int u = u0 + mine + i;
         if (u < nunits) {
-            const int k = u / per_cam;
-            const int rem = u - k * per_cam;
-            const int pp = rem / Nscale;
-            const int sc = rem - pp * Nscale;
             const float2 uv = sloc[pp * Ncam + k];
             const float cs = svn ? svn[k] : 1.0f;
             const MapInfo m = smap[k * Nscale + sc];
@@ -100,13 +102,20 @@ __device__ __forceinline__ int build_unit_list(int u0, int nunits, int P, int Nc
                 r.W = m.W;
                 r.fx = c.fx;
                 r.fy = c.fy;
-                r.wf = ((((pp * Ncam + k) * Nscale) + sc) << 4) | (c.x0 >= 0 ? 1 : 0) | (c.x0 + 1 < m.W ? 2 : 0) |
+                r.wf = ((((pp * pitch + k) * Nscale) + sc) << 4) | (c.x0 >= 0 ? 1 : 0) | (c.x0 + 1 < m.W ? 2 : 0) |
                        (c.y0 >= 0 ? 4 : 0) | (c.y0 + 1 < m.H ? 8 : 0);
-                r.scale = cs;
+                r.scale = svn ? cs : __int_as_float(u);
                 ul.rec[mine + i] = r;
                 vmask |= 1u << i;
             } else {
-                dropped(pp, k, sc);
+                dropped((pp * pitch + k) * Nscale + sc);
+            }
+        }
+        if (++sc == Nscale) {
+            sc = 0;
+            if (++pp == P) {
+                pp = 0;
+                ++k;
             }
         }
     }
