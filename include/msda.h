@@ -122,6 +122,15 @@ typedef struct {
  * write every row. */
 #define MSDA_FLAG_GRAD_FEAT_ZEROED 1
 
+/* tuning->flags: the deterministic msda_backward writes grad_feat in the
+ * type of feat (grad_feat then points to [B, sum_hw, C] elements of
+ * feat_dtype), each element the FP32 sum rounded once, to nearest even: what
+ * a caller that wants the gradient in the features' type would get by
+ * converting the FP32 gradient, without writing and reading that.  With the
+ * atomic mode or tuning->variant = 2 and a reduced-precision feat the call
+ * returns MSDA_ERR_UNSUPPORTED; with FP32 features it changes nothing. */
+#define MSDA_FLAG_GRAD_FEAT_IN_FEAT_TYPE 2
+
 /* ------------------------------------------------------------------------
  * msda_forward - the operator above (Sec. 3.2 multi-scale multi-view
  * feature extraction at projected keypoints; Sec. 5.3 MSDA).

@@ -283,6 +283,12 @@ msda_status msda_backward(const void* feat, msda_dtype feat_dtype, const int32_t
     if (p.C % 4 != 0) return fail(MSDA_ERR_UNSUPPORTED, "msda_backward: C must be a multiple of 4");
     prefer_split(tuning, &p, 2);
     const int warps = pick_warps(tuning, 4);
+    if (tuning && (tuning->flags & MSDA_FLAG_GRAD_FEAT_IN_FEAT_TYPE) && feat_dtype != MSDA_F32) {
+        if (!deterministic || tuning->variant == 2)
+            return fail(MSDA_ERR_UNSUPPORTED, "msda_backward: grad_feat in feat's type needs the deterministic mode, "
+                        "not its staged form");
+        p.gf_t = feat_dtype;
+    }
     if (deterministic) {
         if (workspace && !aligned16(workspace))
             return fail(MSDA_ERR_WORKSPACE, "msda_backward: workspace must be 256-byte aligned");

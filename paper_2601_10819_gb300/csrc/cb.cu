@@ -147,7 +147,8 @@ struct CbArgs {
     const float* loc;
     const void* w;
     const float* go;
-    float* gfeat;
+    void* gfeat;
+    int gf_t;  // msda_dtype of gfeat
     unsigned char* ws;
     CbLayout L;
     int B, sum_hw, C, Ncam, Nscale, nmaps, A, P, G, Cg;
@@ -377,8 +378,14 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
             const int2 gp = gaps[gi];
             const long long n = (long long)(gp.y - gp.x) * c4;
             for (int b = 0; b < a.B && n > 0; ++b) {
-                float4* dst = reinterpret_cast<float4*>(a.gfeat + ((long long)b * a.sum_hw + gp.x) * a.C);
-                for (long long i = threadIdx.x; i < n; i += blockDim.x) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                const long long first = ((long long)b * a.sum_hw + gp.x) * c4;  // in groups of four channels
+                if (a.gf_t == MSDA_F32) {
+                    float4* dst = reinterpret_cast<float4*>(a.gfeat) + first;
+                    for (long long i = threadIdx.x; i < n; i += blockDim.x) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                } else {
+                    uint2* dst = reinterpret_cast<uint2*>(a.gfeat) + first;
+                    for (long long i = threadIdx.x; i < n; i += blockDim.x) dst[i] = make_uint2(0u, 0u);
+                }
             }
         }
         return;
@@ -605,7 +612,9 @@ __global__ void __launch_bounds__(256) cb_loc_kernel(const CbArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// Row reduce as column sweeps.  Block j works on channel group g = j % G: it stages grad_out[b, :, group g] in
+// Row reduce as column sweeps (grad_feat in FP32, or narrowed once in the features' type: the row's sum is in
+// registers either way, and a caller that wants the narrow gradient saves writing and reading the FP32 one; 16 cameras,
+// batch 4, BF16: a 205 us conversion after a 732 us reduce, against a 734 us reduce alone).  Block j works on channel group g = j % G: it stages grad_out[b, :, group g] in
 // shared memory for b = 0, 1, ... in turn and takes whole maps of (b, g) from that pair's queue.  A map's
 // columns, cut into row segments, are swept top to bottom: at cell row cy a column j reads the records of its
 // two cells (cy, j-1) and (cy, j), which are adjacent in record order, and adds each record once to the row it
@@ -634,6 +643,18 @@ __device__ __forceinline__ void cb_fma2x2(float4& cur, float4& nxt, float kc, fl
     n1 = __ffma2_rn(knn, vb, n1);
     cur = make_float4(c0.x, c0.y, c1.x, c1.y);
     nxt = make_float4(n0.x, n0.y, n1.x, n1.y);
+}
+
+// Elements of grad_feat: FP32, or (LOWP) 16 bits in the features' type.
+template <bool LOWP> struct GradElem { using T = float; };
+template <> struct GradElem<true> { using T = unsigned short; };
+
+// Store four channels of a feature row's gradient.
+__device__ __forceinline__ void cb_store(const CbArgs&, float* dst, const float4& v) {
+    *reinterpret_cast<float4*>(dst) = v;
+}
+__device__ __forceinline__ void cb_store(const CbArgs& a, unsigned short* dst, const float4& v) {
+    *reinterpret_cast<uint2*>(dst) = narrow4(v, a.gf_t == MSDA_F16);
 }
 
 // One cell row of a column from a staged band: records [e, e2) (record e is coefficient slot e - ce and anchor-offset
@@ -711,8 +732,9 @@ __device__ __forceinline__ CbBand cb_issue_band(const CbArgs& a, unsigned char* 
 // records, anchor offsets and cell pointers taken from the workspace (record e, anchor offset e, cell pointer c
 // at their own indices).  Kept out of line so the staged sweep, which nearly every band takes, is compiled
 // as if it were alone.
+template <typename GT>
 __device__ __noinline__ void cb_sweep_in_place(const CbArgs& a, const float4* __restrict__ coef_g,
-                                               const float4* __restrict__ sgo, float* gfm, long long pm, int i0,
+                                               const float4* __restrict__ sgo, GT* gfm, long long pm, int i0,
                                                int i1, int W, int seg, int ntask, int l, int t0, int tstep, bool failed) {
     const int W1 = W + 1;
     const uint32_t* Ao = reinterpret_cast<const uint32_t*>(a.ws + a.L.aoff);
@@ -730,7 +752,7 @@ __device__ __noinline__ void cb_sweep_in_place(const CbArgs& a, const float4* __
                 cb_step<true>(Ao, coef_g, sgo, l, q0, q1, q2, 0u, 0u, cur, nxt);
             } else {
                 cb_step<false>(Ao, coef_g, sgo, l, q0, q1, q2, 0u, 0u, cur, nxt);
-                *reinterpret_cast<float4*>(gfm + ((long long)cy * W + j) * a.C) = cur;
+                cb_store(a, gfm + ((long long)cy * W + j) * a.C, cur);
             }
             cur = nxt;
             nxt = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -758,9 +780,9 @@ __device__ __noinline__ void cb_sweep_in_place(const CbArgs& a, const float4* __
 // passes to start; at 13 a warp per cell takes 150 us against 130 us for a lane group, at 44 79 against 86 us, and
 // where keypoints crowd (projected, 17x30, 21 per cell on average) 88 against 132 us, since a warp evens out its cells.
 // ---------------------------------------------------------------------------
-template <int LG>
+template <int LG, typename GT>
 __device__ __noinline__ int cb_dense_map(const CbArgs& a, const float4* __restrict__ coef_g,
-                                         const float4* __restrict__ sgo, float4* scratch, int ncap, float* gfm,
+                                         const float4* __restrict__ sgo, float4* scratch, int ncap, GT* gfm,
                                          long long pm, int H, int W, uint32_t* cptr, int* ctr, int* fail, uint64_t* mbar,
                                          uint32_t ph0, uint32_t ph1, bool by_warp) {
     constexpr int NLGW = 32 / LG;
@@ -902,18 +924,19 @@ __device__ __noinline__ int cb_dense_map(const CbArgs& a, const float4* __restri
             const float4* up = scratch + ((long long)((i % (R + 1)) * W1 + j) * 4) * LG + l;
             const float4* dn = scratch + ((long long)(((i + 1) % (R + 1)) * W1 + j) * 4) * LG + l;
             const float4 x3 = up[3 * LG], x2 = up[(4 + 2) * LG], x1 = dn[1 * LG], x0 = dn[4 * LG];
-            *reinterpret_cast<float4*>(gfm + ((long long)i * W + j) * a.C) =
-                make_float4(x3.x + x2.x + x1.x + x0.x, x3.y + x2.y + x1.y + x0.y, x3.z + x2.z + x1.z + x0.z,
-                            x3.w + x2.w + x1.w + x0.w);
+            cb_store(a, gfm + ((long long)i * W + j) * a.C,
+                     make_float4(x3.x + x2.x + x1.x + x0.x, x3.y + x2.y + x1.y + x0.y, x3.z + x2.z + x1.z + x0.z,
+                                 x3.w + x2.w + x1.w + x0.w));
         }
         __syncthreads();
     }
     return npass;
 }
 
-template <int LG>
+template <int LG, bool LOWP>
 __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a) {
     constexpr int NLGW = 32 / LG;  // lane groups per warp
+    using GT = typename GradElem<LOWP>::T;
     const CbHeader* hdr = reinterpret_cast<const CbHeader*>(a.ws);
     if (!hdr->ok) return;
     const int ngb = gridDim.x / a.G;
@@ -954,7 +977,7 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
         int* queue = queues + b * a.G + g;
         if (threadIdx.x == 0) s_item[0] = atomicAdd(queue, 1);
         __syncthreads();
-        float* gfb = a.gfeat + (long long)b * a.sum_hw * a.C + g * a.Cg + l * 4;
+        GT* gfb = reinterpret_cast<GT*>(a.gfeat) + (long long)b * a.sum_hw * a.C + g * a.Cg + l * 4;
         for (int cur_slot = 0;; cur_slot ^= 1) {
             const int m = s_item[cur_slot];
             if (m >= a.nmaps) break;
@@ -963,12 +986,12 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
             if (mp.W != 0) {
                 const int H = mp.H, W = mp.W, W1 = W + 1;
                 const long long pm = (long long)b * a.L.nccap + mp.cbase;  // the map's cell pointers
-                float* gfm = gfb + (long long)mp.start * a.C;
+                GT* gfm = gfb + (long long)mp.start * a.C;
                 // a dense map takes its cells one by one, if the corner sums of two cell rows fit in the band buffers
                 const int ncap = min((int)(2 * L.bsize / (4 * sizeof(float) * (size_t)a.Cg)), kCbDensePtrs - 8);
                 const uint32_t nrec = __ldg(cellptr + pm + (long long)(H + 1) * W1) - __ldg(cellptr + pm);
                 if (nrec >= (uint32_t)kCbDensePerRow * (uint32_t)(H * W) && 2 * W1 <= ncap) {
-                    const int npass = cb_dense_map<LG>(a, coef_g, sgo, reinterpret_cast<float4*>(buf0), ncap, gfm, pm, H, W, rp, &s_ctr,
+                    const int npass = cb_dense_map<LG, GT>(a, coef_g, sgo, reinterpret_cast<float4*>(buf0), ncap, gfm, pm, H, W, rp, &s_ctr,
                                      &s_fail, mbar, ph0, ph1,
                                      nrec >= (uint32_t)kCbWarpPerCell * (uint32_t)((H + 1) * W1));
                     ph0 ^= (uint32_t)((npass + 1) / 2) & 1u;  // the passes took the two barriers in turn
@@ -1035,7 +1058,7 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
                     const int ntask = W * S;
                     const bool failed = s_fail != 0;
                     if (direct) {
-                        cb_sweep_in_place(a, coef_g, sgo, gfm, pm, i0, i1, W, seg, ntask, l, lgid, nlg, failed);
+                        cb_sweep_in_place<GT>(a, coef_g, sgo, gfm, pm, i0, i1, W, seg, ntask, l, lgid, nlg, failed);
                     } else {
                         const float4* Cf = reinterpret_cast<const float4*>(bb);
                         const uint32_t* Ao = reinterpret_cast<const uint32_t*>(bb + L.aoff);
@@ -1054,7 +1077,7 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
                                     cb_step<true>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, cur, nxt);
                                 } else {
                                     cb_step<false>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, cur, nxt);
-                                    *reinterpret_cast<float4*>(gfm + ((long long)cy * W + j) * a.C) = cur;
+                                    cb_store(a, gfm + ((long long)cy * W + j) * a.C, cur);
                                 }
                                 cur = nxt;
                                 nxt = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1077,14 +1100,15 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
 using CbBinKernel = void (*)(const CbArgs);
 using CbRedKernel = void (*)(const CbArgs);
 
+template <bool LOWP>
 static CbRedKernel cb_red_pick(int lg) {
     switch (lg) {
-        case 1: return cb_reduce_kernel<1>;
-        case 2: return cb_reduce_kernel<2>;
-        case 4: return cb_reduce_kernel<4>;
-        case 8: return cb_reduce_kernel<8>;
-        case 16: return cb_reduce_kernel<16>;
-        case 32: return cb_reduce_kernel<32>;
+        case 1: return cb_reduce_kernel<1, LOWP>;
+        case 2: return cb_reduce_kernel<2, LOWP>;
+        case 4: return cb_reduce_kernel<4, LOWP>;
+        case 8: return cb_reduce_kernel<8, LOWP>;
+        case 16: return cb_reduce_kernel<16, LOWP>;
+        case 32: return cb_reduce_kernel<32, LOWP>;
     }
     return nullptr;
 }
@@ -1097,7 +1121,7 @@ msda_status launch_backward_cb(const Problem& p, const float* grad_out, float* g
     msda_status st = device_info(&dev);
     if (st != MSDA_OK) return st;
     CbArgs a;
-    a.shape = p.shape; a.start = p.start; a.loc = p.loc; a.w = p.w; a.go = grad_out; a.gfeat = grad_feat;
+    a.shape = p.shape; a.start = p.start; a.loc = p.loc; a.w = p.w; a.go = grad_out; a.gfeat = grad_feat; a.gf_t = p.gf_t;
     a.ws = reinterpret_cast<unsigned char*>(ws);
     a.L = cb_layout(p, body_base);
     a.B = p.B; a.sum_hw = p.sum_hw; a.C = p.C; a.Ncam = p.Ncam; a.Nscale = p.Nscale; a.nmaps = p.Ncam * p.Nscale;
@@ -1108,7 +1132,7 @@ msda_status launch_backward_cb(const Problem& p, const float* grad_out, float* g
     a.status = dev.status;
     CbBinKernel bin = p.w_t == MSDA_F32 ? cb_bin_kernel<float>
                     : p.w_t == MSDA_BF16 ? cb_bin_kernel<__nv_bfloat16> : cb_bin_kernel<__half>;
-    CbRedKernel red = cb_red_pick(p.Cg / 4);
+    CbRedKernel red = p.gf_t == MSDA_F32 ? cb_red_pick<false>(p.Cg / 4) : cb_red_pick<true>(p.Cg / 4);
     if (!red) return fail(MSDA_ERR_UNSUPPORTED, "msda_backward: no cell-binned reduce for C/G = %d", p.Cg);
     const size_t bin_smem = (size_t)a.bin_smem;
     const size_t red_smem = CbRedSmem(p.A, p.Cg, a.nb).total;

@@ -95,6 +95,21 @@ __device__ __forceinline__ void store_out(float* o, float v) { *o = v; }
 __device__ __forceinline__ void store_out(__nv_bfloat16* o, float v) { *o = __float2bfloat16_rn(v); }
 __device__ __forceinline__ void store_out(__half* o, float v) { *o = __float2half_rn(v); }
 
+// Four consecutive values of a row narrowed to BF16 or FP16 (RNE), as 8 bytes.
+__device__ __forceinline__ uint2 narrow4(const float4& v, bool half) {
+    uint2 r;
+    if (half) {
+        const __half2 a = __floats2half2_rn(v.x, v.y), b = __floats2half2_rn(v.z, v.w);
+        r.x = *reinterpret_cast<const uint32_t*>(&a);
+        r.y = *reinterpret_cast<const uint32_t*>(&b);
+    } else {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        r.x = *reinterpret_cast<const uint32_t*>(&a);
+        r.y = *reinterpret_cast<const uint32_t*>(&b);
+    }
+    return r;
+}
+
 // ---------------------------------------------------------------------------
 // Projected location -> bilinear cell.
 //

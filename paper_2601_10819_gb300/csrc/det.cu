@@ -404,7 +404,8 @@ struct RedArgs {
     const uint32_t* e_pt;    //   point-scale index (t * Nscale + s)
     const uint32_t* e_ba;    //   anchor row b * A + a of grad_out
     int wide;                // grad_out rows and lane chunks 32-byte aligned: 256-bit loads
-    float* gfeat;
+    void* gfeat;
+    int gf_t;                // msda_dtype of gfeat
     long long nrows;
     int sum_hw, C, Ncam, Nscale, A, P, G, Cg, rt, sbits;
     FastDiv ncam, pncam;  // divisions by Ncam and P*Ncam
@@ -497,9 +498,13 @@ __global__ void __launch_bounds__(256) det_reduce_kernel(const RedArgs a) {
             }
         }
     }
-    float4* dst = reinterpret_cast<float4*>(a.gfeat + row * a.C + c0);
+    const long long d0 = (row * a.C + c0) / 4;  // in groups of four channels
 #pragma unroll
-    for (int j = 0; j < CPL / 4; ++j) dst[j] = make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+    for (int j = 0; j < CPL / 4; ++j) {
+        const float4 v = make_float4(acc[4 * j], acc[4 * j + 1], acc[4 * j + 2], acc[4 * j + 3]);
+        if (a.gf_t == MSDA_F32) reinterpret_cast<float4*>(a.gfeat)[d0 + j] = v;
+        else reinterpret_cast<uint2*>(a.gfeat)[d0 + j] = narrow4(v, a.gf_t == MSDA_F16);
+    }
     }
 }
 
@@ -691,7 +696,7 @@ msda_status launch_backward_det(const Problem& p, const float* grad_out, float* 
     sl.ntiles = L.ntiles;
     RedArgs& ra = sl.ra;
     ra.shape = p.shape; ra.start = p.start; ra.loc = p.loc; ra.w = p.w; ra.go = grad_out;
-    ra.vals = sl.vals; ra.rowptr = sl.rowptr; ra.gfeat = grad_feat; ra.nrows = nrows;
+    ra.vals = sl.vals; ra.rowptr = sl.rowptr; ra.gfeat = grad_feat; ra.gf_t = p.gf_t; ra.nrows = nrows;
     ra.e_om = reinterpret_cast<const float*>(sl.e_om);
     ra.e_pt = sl.e_pt;
     ra.e_ba = sl.e_ba;

@@ -22,6 +22,7 @@ struct Problem {
     int Cg;  // channels per group
     int nv;  // 16-byte chunks per lane (1, 2 or 4)
     int rt;  // lanes per channel row (power of two, <= 32)
+    msda_dtype gf_t = MSDA_F32;  // type the deterministic backward writes grad_feat in (MSDA_F32 or feat_t)
 };
 
 struct DeviceInfo {

@@ -45,6 +45,7 @@ class msda_tuning(ctypes.Structure):
 
 
 FLAG_GRAD_FEAT_ZEROED = 1
+FLAG_GRAD_FEAT_IN_FEAT_TYPE = 2
 
 
 class msda_scene(ctypes.Structure):
@@ -267,7 +268,7 @@ def backward(feat, spatial_shape, scale_start_index, sampling_location, weights,
     workspace: allocated when None (or, in deterministic mode, too small).  In
     atomic mode a caller's workspace is passed through as is: one of fewer
     than 8 bytes selects the static-stride item order.
-    flags: extra MSDA_FLAG_* bits.
+    flags: extra MSDA_FLAG_* bits; with FLAG_GRAD_FEAT_IN_FEAT_TYPE, grads[0] is a tensor of feat's type.
     """
     lib = load()
     B, sum_hw, C, Ncam, Nscale, A, P, G = _dims(feat, spatial_shape, scale_start_index, sampling_location, weights)
@@ -419,8 +420,8 @@ def plan_batched(scenes: Sequence, out_dtype: torch.dtype = torch.float32, warps
 class MSDAFunction(torch.autograd.Function):
     """Differentiable MSDA: gradients for feat, sampling_location and weights.
 
-    The forward output is float32; the gradients are float32 and are cast to
-    the input dtypes when those are reduced precision.  The backward is the
+    The forward output is float32; the gradients are computed in float32 and
+    rounded once to the input dtypes when those are reduced precision.  The backward is the
     deterministic mode unless deterministic=False (the atomic mode).
     """
 
@@ -434,8 +435,14 @@ class MSDAFunction(torch.autograd.Function):
     @staticmethod
     def backward(ctx, grad_out):
         feat, shape, start, loc, w = ctx.saved_tensors
+        grads, flags = None, 0
+        if ctx.deterministic and feat.dtype != torch.float32:
+            # the feature gradient is rounded once either way: written in feat's type by the kernel
+            grads = (torch.empty_like(feat), torch.empty_like(loc),
+                     torch.empty(w.shape, dtype=torch.float32, device=w.device))
+            flags = FLAG_GRAD_FEAT_IN_FEAT_TYPE
         gf, gl, gw = backward(feat, shape, start, loc, w, grad_out.contiguous().float(),
-                              deterministic=ctx.deterministic)
+                              deterministic=ctx.deterministic, grads=grads, flags=flags)
         return (gf.to(feat.dtype) if ctx.needs_input_grad[0] else None, None, None,
                 gl if ctx.needs_input_grad[3] else None,
                 gw.to(w.dtype) if ctx.needs_input_grad[4] else None, None)
