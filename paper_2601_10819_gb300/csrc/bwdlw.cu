@@ -22,7 +22,9 @@
 // together read the maps of the same few cameras, and there are enough of them that the last wave is
 // short and that few anchors still fill the GPU.  Alone on the GPU, 64
 // cameras of 1080p maps, 4 warps: 900 anchors 695 -> 397 us, 100 anchors
-// 355 -> 80 us (one block per anchor and all its cameras before).  The
+// 355 -> 80 us (one block per anchor and all its cameras before); with the
+// weights' lines fetched ahead, as in fwd.cu, inside the step 393 -> 379 us and
+// 540 -> 511 us for 16 cameras of batch 4.  The
 // latency of the corner rows bounds it (3.5 GB from L2, 180 us at the probed
 // gather rate), with three blocks of 8 warps, or six of 4, per SM.  A camera
 // whose locations and sums do not fit in shared memory falls back to the per-point kernel of bwd.cu without its scatter.
@@ -155,7 +157,8 @@ __global__ void __launch_bounds__(256, NV == 2 ? 3 : (NV == 1 ? 4 : 2)) bwd_locw
                                               } else {
                                                   for (int gg = 0; gg < G; ++gg) d[gg] = 0.0f;
                                               }
-                                          });
+                                          },
+                                          [&](int row) { prefetch_line(wb + (long long)row * G); });
         for (int q = team; q < total; q += nteams) {
             const UnitRec r = ul.rec[ul.list[q]];
             const int ps = r.wf >> 4;  // (pp * Ncam + k) * Nscale + s

@@ -44,6 +44,11 @@ __device__ __forceinline__ void ld32(const void* p, uint4& lo, uint4& hi) {
                  : "l"(p));
 }
 
+// Start fetching the line of p into L2.
+__device__ __forceinline__ void prefetch_line(const void* p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(p)) : "memory");
+}
+
 // Widen the VEC channels of one 16-byte chunk to FP32.
 __device__ __forceinline__ void widen(const uint4& v, float* f, float) {
     f[0] = __uint_as_float(v.x); f[1] = __uint_as_float(v.y);

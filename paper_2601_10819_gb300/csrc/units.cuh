@@ -75,12 +75,13 @@ struct UnitList {
 // Stage A for the chunk starting at u0: returns the number of listed point-scales (the same in every thread).
 // A point-scale's weights are row (pp * pitch + k) * Nscale + s of the caller's (pitch: cameras between two keypoints,
 // Ncam unless the caller's cameras are a slice).  dropped(row) is called, by the thread that owns it, for each
-// point-scale of the chunk that is not listed.  Ends with a block barrier, so the list is ready for stage B.
-template <typename Dropped>
+// point-scale of the chunk that is not listed, and listed(row) for the first one of each thread that is (to fetch its
+// weights' line ahead).  Ends with a block barrier, so the list is ready for stage B.
+template <typename Dropped, typename Listed>
 __device__ __forceinline__ int build_unit_list(int u0, int nunits, int P, int Ncam, int Nscale, int pitch,
                                                const MapInfo* __restrict__ smap, const float4* __restrict__ sbox,
                                                const float2* __restrict__ sloc, const float* __restrict__ svn,
-                                               const UnitList& ul, Dropped dropped) {
+                                               const UnitList& ul, Dropped dropped, Listed listed) {
     const int per_cam = P * Nscale;
     const int mine = (int)threadIdx.x * kUnitsPerThread;
     unsigned vmask = 0u;
@@ -119,6 +120,7 @@ __device__ __forceinline__ int build_unit_list(int u0, int nunits, int P, int Nc
             }
         }
     }
+    if (vmask) listed(ul.rec[mine + __ffs(vmask) - 1].wf >> 4);
     int off = block_excl_scan(__popc(vmask), ul.scan, ul.scan + 8);
 #pragma unroll
     for (int i = 0; i < kUnitsPerThread; ++i)
