@@ -5,7 +5,9 @@
 #include <stdarg.h>
 #include <stdio.h>
 
+#include <map>
 #include <mutex>
+#include <utility>
 
 #include "common.cuh"
 #include "internal.h"
@@ -58,8 +60,15 @@ msda_status ensure_smem(const void* func, size_t bytes, const DeviceInfo& dev) {
         return fail(MSDA_ERR_UNSUPPORTED, "needs %zu bytes of shared memory per block (limit %d)", bytes,
                     dev.max_smem_optin);
     if (bytes <= 48 * 1024) return MSDA_OK;
+    // The limit set last per kernel and device: raised only when a call needs more (about 1 us a call otherwise).
+    static std::mutex mu;
+    static std::map<std::pair<const void*, int>, size_t> limit;
+    std::lock_guard<std::mutex> lock(mu);
+    size_t& have = limit[{func, dev.device}];
+    if (bytes <= have) return MSDA_OK;
     const cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return fail(MSDA_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
+    have = bytes;
     return MSDA_OK;
 }
 

@@ -604,6 +604,11 @@ static SideStream* side_stream(int device, bool may_create) {
     return g_side_state[device] == 1 ? &g_side[device] : nullptr;
 }
 
+// Point-scales from which the cell-binned kernels go to the side stream.  Below, the kernels take a few microseconds each
+// and the call is bound by its launches: the four event calls cost more than the overlap gives (a step through autograd
+// 252 -> 248 us with 256 point-scales, 253 -> 236 us with 7200; with 33 000, 90 us on two streams against 95 us on one).
+constexpr long long kSideMin = 32768;
+
 msda_status launch_backward_det(const Problem& p, const float* grad_out, float* grad_feat,
                                 float* grad_loc, float* grad_w, void* ws, size_t ws_bytes,
                                 int warps, bool allow_cells, cudaStream_t stream) {
@@ -645,7 +650,7 @@ msda_status launch_backward_det(const Problem& p, const float* grad_out, float* 
     if (cells && cudaStreamIsCapturing(stream, &cap) != cudaSuccess) return check_launch("msda_backward capture query");
     std::unique_lock<std::mutex> side_lock(g_side_mu, std::defer_lock);
     SideStream* side = nullptr;
-    if (cells) {
+    if (cells && npts >= kSideMin) {
         side_lock.lock();
         side = side_stream(dev.device, cap == cudaStreamCaptureStatusNone);
         if (side && (cudaEventRecord(side->fork, stream) != cudaSuccess ||

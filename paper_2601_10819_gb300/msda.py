@@ -62,6 +62,8 @@ def library_path() -> str:
 def load(path: Optional[str] = None):
     """Load the shared library (no build).  Raises if it is missing."""
     global _lib
+    if _lib is not None and path is None:  # set once, after its prototypes
+        return _lib
     with _lock:
         if _lib is not None and path is None:
             return _lib
@@ -111,13 +113,19 @@ def _check(fn: str, rc: int):
         raise MSDAError(fn, rc, _lib.msda_last_error().decode())
 
 
+# The raw stream without a Stream object around it: every call passes here.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(device) -> int:
+    if _raw_stream is not None:
+        return _raw_stream(device.index)
     return torch.cuda.current_stream(device).cuda_stream
 
 
 def _tuning(warps: Optional[int], blocks_per_sm: Optional[int] = None, variant: int = 0, vec: int = 0,
             flags: int = 0):
-    if not warps and not blocks_per_sm and not variant and not vec and not flags:
+    if not (warps or blocks_per_sm or variant or vec or flags):
         return None
     t = msda_tuning()
     t.warps_per_block = int(warps or 0)
@@ -129,16 +137,19 @@ def _tuning(warps: Optional[int], blocks_per_sm: Optional[int] = None, variant: 
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()  # the prototypes make it a void pointer
 
 
 def _dims(feat, spatial_shape, scale_start_index, sampling_location, weights):
-    for name, t in (("feat", feat), ("spatial_shape", spatial_shape), ("scale_start_index", scale_start_index),
-                    ("sampling_location", sampling_location), ("weights", weights)):
-        if not t.is_cuda:
-            raise ValueError(f"{name} must be a CUDA tensor")
-        if not t.is_contiguous():
-            raise ValueError(f"{name} must be contiguous")
+    if not (feat.is_cuda and spatial_shape.is_cuda and scale_start_index.is_cuda and sampling_location.is_cuda and
+            weights.is_cuda and feat.is_contiguous() and spatial_shape.is_contiguous() and
+            scale_start_index.is_contiguous() and sampling_location.is_contiguous() and weights.is_contiguous()):
+        for name, t in (("feat", feat), ("spatial_shape", spatial_shape), ("scale_start_index", scale_start_index),
+                        ("sampling_location", sampling_location), ("weights", weights)):
+            if not t.is_cuda:
+                raise ValueError(f"{name} must be a CUDA tensor")
+            if not t.is_contiguous():
+                raise ValueError(f"{name} must be contiguous")
     if spatial_shape.dtype != torch.int32 or scale_start_index.dtype != torch.int32:
         raise ValueError("spatial_shape and scale_start_index must be int32")
     if sampling_location.dtype != torch.float32:
@@ -147,15 +158,15 @@ def _dims(feat, spatial_shape, scale_start_index, sampling_location, weights):
         raise ValueError("feat/weights must be float32, bfloat16 or float16")
     B, sum_hw, C = feat.shape
     Ncam, Nscale, two = spatial_shape.shape
-    if two != 2 or tuple(scale_start_index.shape) != (Ncam, Nscale):
+    if two != 2 or scale_start_index.shape != (Ncam, Nscale):
         raise ValueError("spatial_shape must be [Ncam, Nscale, 2] and scale_start_index [Ncam, Nscale]")
     B2, A, P, Ncam2, two = sampling_location.shape
     if B2 != B or Ncam2 != Ncam or two != 2:
         raise ValueError("sampling_location must be [B, A, P, Ncam, 2]")
-    if weights.dim() != 6 or tuple(weights.shape[:5]) != (B, A, P, Ncam, Nscale):
+    wshape = weights.shape
+    if len(wshape) != 6 or wshape[:5] != (B, A, P, Ncam, Nscale):
         raise ValueError("weights must be [B, A, P, Ncam, Nscale, G]")
-    G = weights.shape[5]
-    return B, sum_hw, C, Ncam, Nscale, A, P, G
+    return B, sum_hw, C, Ncam, Nscale, A, P, wshape[5]
 
 
 def forward_workspace_size(B, sum_hw, C, Ncam, Nscale, A, P, G) -> int:
@@ -188,7 +199,7 @@ def forward(feat, spatial_shape, scale_start_index, sampling_location, weights, 
     rc = lib.msda_forward(_ptr(feat), _DT[feat.dtype], _ptr(spatial_shape), _ptr(scale_start_index),
                           _ptr(sampling_location), _ptr(weights), _DT[weights.dtype], _ptr(out), _DT[out.dtype],
                           B, sum_hw, C, Ncam, Nscale, A, P, G, _ptr(workspace), ws_bytes, _tuning(warps, None, variant, vec),
-                          ctypes.c_void_p(_stream(feat.device)))
+                          _stream(feat.device))
     _check("msda_forward", rc)
     return out
 
@@ -210,7 +221,7 @@ def forward_train(feat, spatial_shape, scale_start_index, sampling_location, wei
     rc = lib.msda_forward_train(_ptr(feat), _DT[feat.dtype], _ptr(spatial_shape), _ptr(scale_start_index),
                                 _ptr(sampling_location), _ptr(weights), _DT[weights.dtype], _ptr(out), _DT[out.dtype],
                                 _ptr(grad_feat), B, sum_hw, C, Ncam, Nscale, A, P, G,
-                                _tuning(warps, None, variant, vec), ctypes.c_void_p(_stream(feat.device)))
+                                _tuning(warps, None, variant, vec), _stream(feat.device))
     _check("msda_forward_train", rc)
     return out
 
@@ -229,7 +240,7 @@ def forward_oae(feat, spatial_shape, scale_start_index, sampling_location, weigh
     rc = lib.msda_forward_oae(_ptr(feat), _DT[feat.dtype], _ptr(spatial_shape), _ptr(scale_start_index),
                               _ptr(sampling_location), _ptr(weights), _DT[weights.dtype], _ptr(visibility),
                               _ptr(out), _DT[out.dtype], B, sum_hw, C, Ncam, Nscale, A, P, G,
-                              _tuning(warps, None, variant, vec), ctypes.c_void_p(_stream(feat.device)))
+                              _tuning(warps, None, variant, vec), _stream(feat.device))
     _check("msda_forward_oae", rc)
     return out
 
@@ -249,7 +260,7 @@ def keypoints(anchors, offsets, dt, proj, img_wh, *, out: Optional[torch.Tensor]
     if out is None:
         out = torch.empty(B, A, P, Ncam, 2, dtype=torch.float32, device=anchors.device)
     rc = lib.msda_keypoints(_ptr(anchors), _ptr(offsets), _ptr(dt), _ptr(proj), _ptr(img_wh), _ptr(out),
-                            B, A, P, Ncam, ctypes.c_void_p(_stream(anchors.device)))
+                            B, A, P, Ncam, _stream(anchors.device))
     _check("msda_keypoints", rc)
     return out
 
@@ -292,7 +303,7 @@ def backward(feat, spatial_shape, scale_start_index, sampling_location, weights,
                            int(bool(deterministic)), _ptr(workspace), ws_bytes,
                            _tuning(warps, None, variant, vec,
                                    (FLAG_GRAD_FEAT_ZEROED if grad_feat_zeroed else 0) | int(flags)),
-                           ctypes.c_void_p(_stream(dev)))
+                           _stream(dev))
     _check("msda_backward", rc)
     return gf, gl, gw
 
@@ -319,7 +330,7 @@ def probe_read(buf: torch.Tensor, reps: int, blocks: int, rows: int = 0, sink: O
     if sink is None:
         sink = torch.zeros(blocks, dtype=torch.int32, device=buf.device)
     rc = lib.msda_probe_read(_ptr(buf), buf.numel() * buf.element_size(), reps, blocks, rows, _ptr(sink),
-                             ctypes.c_void_p(_stream(buf.device)))
+                             _stream(buf.device))
     _check("msda_probe_read", rc)
     return sink
 
@@ -329,7 +340,7 @@ def probe_reduce(buf: torch.Tensor, reps: int, blocks: int, rows: int):
     lib = load()
     if buf.dtype != torch.float32 or not buf.is_contiguous():
         raise ValueError("probe_reduce needs a contiguous float32 buffer")
-    rc = lib.msda_probe_reduce(_ptr(buf), buf.numel() * 4, reps, blocks, rows, ctypes.c_void_p(_stream(buf.device)))
+    rc = lib.msda_probe_reduce(_ptr(buf), buf.numel() * 4, reps, blocks, rows, _stream(buf.device))
     _check("msda_probe_reduce", rc)
 
 
@@ -369,7 +380,7 @@ class BatchedPlan:
                                       self.Nscale, self.C, self.P, self.G, self.ft, self.wt, self.ot,
                                       _ptr(self.workspace), self.workspace.numel(), _ptr(self.done_ns),
                                       _tuning(self.warps, self.blocks_per_sm, 0, self.vec),
-                                      ctypes.c_void_p(_stream(dev)))
+                                      _stream(dev))
         _check("msda_forward_batched", rc)
         return self.outs
 
