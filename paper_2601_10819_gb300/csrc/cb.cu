@@ -31,7 +31,7 @@ namespace msda {
 
 constexpr int kCbThreads = 1024;     // threads of the bin and reduce blocks
 constexpr int kCbWarps = kCbThreads / 32;
-constexpr int kCbMaxMaps = 4096;     // maps the single-block plan kernel can sort
+constexpr int kCbMaxMaps = 4096;     // maps the plan's block can sort
 constexpr int kCbDensePerRow = 4;    // records per feature row of a map from which its cells are summed one by one
 constexpr int kCbWarpPerCell = 16;   // records per cell of a dense map from which a warp sums a cell, not a lane group
 constexpr unsigned short kNoCell = 0xffffu;
@@ -159,7 +159,7 @@ struct CbArgs {
 };
 
 // ---------------------------------------------------------------------------
-// Plan (one block): validate the maps, check that the valid ones are disjoint, number their cells and work
+// Plan (block 0): validate the maps, check that the valid ones are disjoint, number their cells and work
 // items, list the uncovered row ranges, clear the work queues.
 // ---------------------------------------------------------------------------
 // Exclusive prefix sum over n <= 4 * blockDim.x values (4 consecutive per thread) of v(i); *total = sum.
@@ -201,8 +201,26 @@ __device__ __forceinline__ void plan_scan(int n, F v, int* out, int* wsum, int* 
     __syncthreads();
 }
 
+// Locations camera-major: loct[b, k, i] = loc[b, i, k] with i = a * P + p, one 32 x 32 tile of a batch element.
+__device__ __forceinline__ void cb_transpose_tile(const CbArgs& a, float2 (*tile)[33], int t) {
+    const int ap = a.A * a.P;
+    const int nti = (ap + 31) / 32, ntk = (a.Ncam + 31) / 32;
+    const int i0 = t % nti * 32, k0 = t / nti % ntk * 32, b = t / nti / ntk;
+    const float2* src = reinterpret_cast<const float2*>(a.loc) + (long long)b * ap * a.Ncam;
+    float2* dst = reinterpret_cast<float2*>(a.ws + a.L.loct) + (long long)b * a.Ncam * ap;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    if (i0 + ty < ap && k0 + tx < a.Ncam) tile[ty][tx] = __ldg(src + (long long)(i0 + ty) * a.Ncam + k0 + tx);
+    __syncthreads();
+    if (k0 + ty < a.Ncam && i0 + tx < ap) dst[(long long)(k0 + ty) * ap + i0 + tx] = tile[tx][ty];
+}
+
+// Block 0 makes the plan; the others, which need nothing of it, transpose the locations meanwhile.
 __global__ void __launch_bounds__(kCbThreads) cb_plan_kernel(const CbArgs a) {
     __shared__ unsigned long long key[kCbMaxMaps];
+    if (blockIdx.x > 0) {
+        cb_transpose_tile(a, reinterpret_cast<float2 (*)[33]>(key), (int)blockIdx.x - 1);
+        return;
+    }
     int* tmp = reinterpret_cast<int*>(key);  // scan output, once the sorted keys are no longer read
     __shared__ int wsum[32];
     __shared__ int s_bad, s_nvalid, s_cells;
@@ -587,27 +605,6 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
                             make_float4(v[j] * f00, v[j] * f01, v[j] * f10, v[j] * f11);
             }
         }
-    }
-}
-
-// Locations camera-major: loct[b, k, i] = loc[b, i, k] with i = a * P + p (32 x 32 tiles through shared memory).
-__global__ void __launch_bounds__(256) cb_loc_kernel(const CbArgs a) {
-    const CbHeader* hdr = reinterpret_cast<const CbHeader*>(a.ws);
-    if (!hdr->ok) return;
-    __shared__ float2 tile[32][33];
-    const int ap = a.A * a.P;
-    const int i0 = blockIdx.x * 32, k0 = blockIdx.y * 32, b = blockIdx.z;
-    const float2* src = reinterpret_cast<const float2*>(a.loc) + (long long)b * ap * a.Ncam;
-    float2* dst = reinterpret_cast<float2*>(a.ws + a.L.loct) + (long long)b * a.Ncam * ap;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int r = ty; r < 32; r += 8) {
-        const int i = i0 + r, kk = k0 + tx;
-        if (i < ap && kk < a.Ncam) tile[r][tx] = __ldg(src + (long long)i * a.Ncam + kk);
-    }
-    __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
-        const int kk = k0 + r, i = i0 + tx;
-        if (i < ap && kk < a.Ncam) dst[(long long)kk * ap + i] = tile[tx][r];
     }
 }
 
@@ -1138,11 +1135,8 @@ msda_status launch_backward_cb(const Problem& p, const float* grad_out, float* g
     const size_t red_smem = CbRedSmem(p.A, p.Cg, a.nb).total;
     if ((st = ensure_smem((const void*)bin, bin_smem, dev)) != MSDA_OK) return st;
     if ((st = ensure_smem((const void*)red, red_smem, dev)) != MSDA_OK) return st;
-    cb_plan_kernel<<<1, kCbThreads, 0, stream>>>(a);
-    {
-        const dim3 lg((unsigned)((p.A * p.P + 31) / 32), (unsigned)((p.Ncam + 31) / 32), (unsigned)p.B);
-        cb_loc_kernel<<<lg, 256, 0, stream>>>(a);
-    }
+    const long long tiles = (((long long)p.A * p.P + 31) / 32) * ((p.Ncam + 31) / 32) * p.B;
+    cb_plan_kernel<<<(unsigned)(1 + tiles), kCbThreads, 0, stream>>>(a);
     const long long nbm = (long long)p.B * a.nmaps;
     bin<<<(unsigned)(nbm + 16), kCbThreads, bin_smem, stream>>>(a);
     const int ngb = dev.sm_count / p.G;
