@@ -55,7 +55,8 @@
  *   synchronise, so they may be captured in a CUDA graph, except that the
  *   first call on a device looks up the device status word and reads
  *   device attributes, which should happen before any capture.  The
- *   deterministic msda_backward runs its cell-binned kernels on a second
+ *   deterministic msda_backward, but for small calls, runs its cell-binned
+ *   kernels on a second
  *   stream of the library's (one per device, made by the first such call
  *   outside a capture), forked from `stream` and joined back to it with
  *   events inside the call, so everything enqueued on `stream` afterwards

@@ -463,15 +463,16 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
     const uint32_t recbase = (uint32_t)(((long long)b * a.nmaps + m) * ap);
     {
         uint32_t* gptr = reinterpret_cast<uint32_t*>(a.ws + a.L.cellptr) + (long long)b * a.L.nccap + mp.cbase;
-        const int nw = stable ? kCbWarps : 1;
+        const int sh = stable ? 5 : 0, nw = 1 << sh;  // kCbWarps cursors per cell, or one (shifts: 13 us a block else)
         const int nent = stable ? kCbWarps * cstride - (kCbWarps - 1) : ncell + 1;  // (ncell, 0) ends the order
         const int per = (nent + blockDim.x - 1) / blockDim.x;
         const int c0 = threadIdx.x * per;
         // scan position q is (cell q / nw, warp q % nw), at counter (q % nw) * cstride + q / nw
+        static_assert(kCbWarps == 32, "");
         uint32_t sum = 0u;
         for (int j = 0; j < per && c0 + j < nent; ++j) {
             const int q = c0 + j;
-            sum += cnt[(q % nw) * cstride + q / nw];
+            sum += cnt[(q & (nw - 1)) * cstride + (q >> sh)];
         }
         uint32_t x = sum;
 #pragma unroll
@@ -494,10 +495,10 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
         uint32_t run = x - sum + (warp > 0 ? (uint32_t)wsum[warp - 1] : 0u);
         for (int j = 0; j < per && c0 + j < nent; ++j) {
             const int q = c0 + j;
-            uint32_t* e = cnt + (q % nw) * cstride + q / nw;
+            uint32_t* e = cnt + (q & (nw - 1)) * cstride + (q >> sh);
             const uint32_t v = *e;
             *e = run;
-            if (q % nw == 0) gptr[q / nw] = recbase + run;
+            if ((q & (nw - 1)) == 0) gptr[q >> sh] = recbase + run;
             run += v;
         }
     }

@@ -604,10 +604,12 @@ static SideStream* side_stream(int device, bool may_create) {
     return g_side_state[device] == 1 ? &g_side[device] : nullptr;
 }
 
-// Point-scales from which the cell-binned kernels go to the side stream.  Below, the kernels take a few microseconds each
-// and the call is bound by its launches: the four event calls cost more than the overlap gives (a step through autograd
-// 252 -> 248 us with 256 point-scales, 253 -> 236 us with 7200; with 33 000, 90 us on two streams against 95 us on one).
-constexpr long long kSideMin = 32768;
+// Calls of fewer point-scales and fewer bytes of FP32 feature gradient keep the cell-binned kernels on the caller's
+// stream: their kernels take a few microseconds each, the call is bound by its launches, and the four event calls cost
+// more than the overlap gives (a step through autograd 252 -> 248 us with 256 point-scales, 253 -> 236 us with 7200).
+// With 33 000 point-scales two streams take 90 us and one 95 us, and with 13 000 over maps of 33 MB of gradient 71 and
+// 81 us.
+constexpr long long kSideMinPoints = 32768, kSideMinBytes = 4 << 20;
 
 msda_status launch_backward_det(const Problem& p, const float* grad_out, float* grad_feat,
                                 float* grad_loc, float* grad_w, void* ws, size_t ws_bytes,
@@ -650,7 +652,7 @@ msda_status launch_backward_det(const Problem& p, const float* grad_out, float* 
     if (cells && cudaStreamIsCapturing(stream, &cap) != cudaSuccess) return check_launch("msda_backward capture query");
     std::unique_lock<std::mutex> side_lock(g_side_mu, std::defer_lock);
     SideStream* side = nullptr;
-    if (cells && npts >= kSideMin) {
+    if (cells && (npts >= kSideMinPoints || 4 * nrows * p.C >= kSideMinBytes)) {
         side_lock.lock();
         side = side_stream(dev.device, cap == cudaStreamCaptureStatusNone);
         if (side && (cudaEventRecord(side->fork, stream) != cudaSuccess ||
