@@ -463,7 +463,7 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
     const uint32_t recbase = (uint32_t)(((long long)b * a.nmaps + m) * ap);
     {
         uint32_t* gptr = reinterpret_cast<uint32_t*>(a.ws + a.L.cellptr) + (long long)b * a.L.nccap + mp.cbase;
-        const int sh = stable ? 5 : 0, nw = 1 << sh;  // kCbWarps cursors per cell, or one (shifts: 13 us a block else)
+        const int sh = stable ? 5 : 0, nw = 1 << sh;  // kCbWarps cursors per cell, or one
         const int nent = stable ? kCbWarps * cstride - (kCbWarps - 1) : ncell + 1;  // (ncell, 0) ends the order
         const int per = (nent + blockDim.x - 1) / blockDim.x;
         const int c0 = threadIdx.x * per;
