@@ -131,10 +131,10 @@ def split_step(sub, grad_out, forward, backward, group=None):
 
 def backward_launches(det, zeroed=False):
     """Kernels msda_backward enqueues on the benchmark frame: atomic: the scatter kernel (and a memset unless
-    the forward cleared grad_feat); deterministic: the cell-binned plan, location transpose, binning and reduce,
+    the forward cleared grad_feat); deterministic: the cell-binned plan (with the location transpose), binning and reduce,
     dloc/dw, and the one-thread launcher that issues the corner-slot form from the device only when the
     cell-binned plan has cleared its flag (it does not on this frame)."""
-    return 6 if det else (1 if zeroed else 2)
+    return 5 if det else (1 if zeroed else 2)
 
 
 def peaks():
