@@ -269,29 +269,45 @@ def backward_workspace_size(B, sum_hw, C, Ncam, Nscale, A, P, G, deterministic: 
     return int(load().msda_backward_workspace_size(B, sum_hw, C, Ncam, Nscale, A, P, G, int(bool(deterministic))))
 
 
+def _check_grad(name, t, dtype, numel, device):
+    """The kernels write numel elements of dtype at t's address: refuse a buffer that they would not fit."""
+    if t is None:  # the library refuses NULL where it would write
+        return
+    reached = t.device == device or t.is_cuda or t.is_pinned()
+    if t.dtype != dtype or not reached or not t.is_contiguous() or t.numel() < numel:
+        raise ValueError(f"{name} must be a contiguous {dtype} tensor of at least {numel} elements that {device} reaches")
+
+
 def backward(feat, spatial_shape, scale_start_index, sampling_location, weights, grad_out, *,
              deterministic: bool = False, workspace: Optional[torch.Tensor] = None,
              grads=None, warps: Optional[int] = None, variant: int = 0, vec: int = 0,
              grad_feat_zeroed: bool = False, flags: int = 0):
-    """msda_backward: (grad_feat, grad_loc, grad_weights), all float32.
+    """msda_backward: (grad_feat, grad_loc, grad_weights), float32 (grad_feat in feat's type under
+    FLAG_GRAD_FEAT_IN_FEAT_TYPE).
 
+    grads: buffers for the three, allocated when None; each contiguous, reached by feat's device, of the type
+    that is written and with at least its gradient's elements (a larger one is filled from its start).
     grad_feat_zeroed: the caller already cleared grads[0] (atomic mode only).
     workspace: allocated when None (or, in deterministic mode, too small).  In
     atomic mode a caller's workspace is passed through as is: one of fewer
     than 8 bytes selects the static-stride item order.
-    flags: extra MSDA_FLAG_* bits; with FLAG_GRAD_FEAT_IN_FEAT_TYPE, grads[0] is a tensor of feat's type.
+    flags: extra MSDA_FLAG_* bits.
     """
     lib = load()
     B, sum_hw, C, Ncam, Nscale, A, P, G = _dims(feat, spatial_shape, scale_start_index, sampling_location, weights)
     if grad_out.dtype != torch.float32 or not grad_out.is_contiguous() or tuple(grad_out.shape) != (B, A, C):
         raise ValueError("grad_out must be a contiguous float32 [B, A, C] tensor")
     dev = feat.device
+    gf_dtype = feat.dtype if int(flags) & FLAG_GRAD_FEAT_IN_FEAT_TYPE else torch.float32
     if grads is None:
-        gf = torch.empty(B, sum_hw, C, dtype=torch.float32, device=dev)
+        gf = torch.empty(B, sum_hw, C, dtype=gf_dtype, device=dev)
         gl = torch.empty(B, A, P, Ncam, 2, dtype=torch.float32, device=dev)
         gw = torch.empty(B, A, P, Ncam, Nscale, G, dtype=torch.float32, device=dev)
     else:
         gf, gl, gw = grads
+        _check_grad("grads[0]", gf, gf_dtype, B * sum_hw * C, dev)
+        _check_grad("grads[1]", gl, torch.float32, B * A * P * Ncam * 2, dev)
+        _check_grad("grads[2]", gw, torch.float32, B * A * P * Ncam * Nscale * G, dev)
     need = backward_workspace_size(B, sum_hw, C, Ncam, Nscale, A, P, G, deterministic)
     small = workspace is not None and workspace.numel() * workspace.element_size() < need
     if need and (workspace is None or (small and deterministic)):
@@ -446,14 +462,10 @@ class MSDAFunction(torch.autograd.Function):
     @staticmethod
     def backward(ctx, grad_out):
         feat, shape, start, loc, w = ctx.saved_tensors
-        grads, flags = None, 0
-        if ctx.deterministic and feat.dtype != torch.float32:
-            # the feature gradient is rounded once either way: written in feat's type by the kernel
-            grads = (torch.empty_like(feat), torch.empty_like(loc),
-                     torch.empty(w.shape, dtype=torch.float32, device=w.device))
-            flags = FLAG_GRAD_FEAT_IN_FEAT_TYPE
+        # the feature gradient is rounded once either way: written in feat's type by the deterministic kernels
+        flags = FLAG_GRAD_FEAT_IN_FEAT_TYPE if ctx.deterministic and feat.dtype != torch.float32 else 0
         gf, gl, gw = backward(feat, shape, start, loc, w, grad_out.contiguous().float(),
-                              deterministic=ctx.deterministic, grads=grads, flags=flags)
+                              deterministic=ctx.deterministic, flags=flags)
         return (gf.to(feat.dtype) if ctx.needs_input_grad[0] else None, None, None,
                 gl if ctx.needs_input_grad[3] else None,
                 gw.to(w.dtype) if ctx.needs_input_grad[4] else None, None)
