@@ -32,8 +32,6 @@ namespace msda {
 constexpr int kCbThreads = 1024;     // threads of the bin and reduce blocks
 constexpr int kCbWarps = kCbThreads / 32;
 constexpr int kCbMaxMaps = 4096;     // maps the plan's block can sort
-constexpr int kCbDensePerRow = 4;    // records per feature row of a map from which its cells are summed one by one
-constexpr int kCbWarpPerCell = 16;   // records per cell of a dense map from which a warp sums a cell, not a lane group
 constexpr unsigned short kNoCell = 0xffffu;
 constexpr int kCbMaxBin = 256;       // points of a cell that a warp sorts in registers
 // Cells of a map whose fuller cells are put in order by reading all points again (a larger map with such a cell hands
@@ -57,7 +55,8 @@ struct CbHeader {
 };
 
 struct CbLayout {
-    size_t maps, gaps, queues, plan_end;  // plan area (read by the corner-slot kernels: header.ok)
+    size_t maps, gaps, queues, forms, plan_end;  // plan area (read by the corner-slot kernels: header.ok)
+                                          // forms: per (batch element, map), how the reduce sums it (CbForm)
     size_t cellptr, aoff, coef, loct;     // cell pointers, anchor offsets, per-group corner coefficients,
     size_t total;                         // locations camera-major [B, Ncam, A*P] (float2)
     long long nccap;                      // cell-pointer entries per batch element
@@ -70,7 +69,8 @@ static CbLayout cb_layout(const Problem& p, size_t body_base = 0) {
     L.maps = 256;
     L.gaps = align_up(L.maps + sizeof(CbMap) * (size_t)nmaps, 256);
     L.queues = align_up(L.gaps + sizeof(int2) * (size_t)(nmaps + 1), 256);
-    L.plan_end = align_up(L.queues + sizeof(int) * (size_t)p.B * p.G, 256);
+    L.forms = L.queues + sizeof(int) * (size_t)p.B * p.G;
+    L.plan_end = align_up(L.forms + sizeof(int) * (size_t)p.B * (size_t)nmaps, 256);
     // Disjoint valid maps fit in sum_hw rows, and (H+1)(W+1) + 1 <= 2 H W + 3 for H, W >= 1, so the cell
     // pointers of one batch element need at most 2 sum_hw + 3 Nmaps entries.
     L.nccap = (2ll * p.sum_hw + 3 * nmaps + 3) & ~3ll;  // a multiple of 4: 16-byte aligned batch slices
@@ -152,15 +152,15 @@ struct CbArgs {
     unsigned char* ws;
     CbLayout L;
     int B, sum_hw, C, Ncam, Nscale, nmaps, A, P, G, Cg;
-    int nlg;       // lane groups of a reduce block (light sweep tasks run at once)
     int bin_smem;  // dynamic shared memory of a binning block
     int nb;        // band buffer slots of a reduce block
+    int ncap;      // cells whose corner sums they hold
     int* status;
 };
 
 // ---------------------------------------------------------------------------
-// Plan (block 0): validate the maps, check that the valid ones are disjoint, number their cells and work
-// items, list the uncovered row ranges, clear the work queues.
+// Plan (block 0): validate the maps, check that the valid ones are disjoint, number their cells,
+// list the uncovered row ranges, clear the work queues.
 // ---------------------------------------------------------------------------
 // Exclusive prefix sum over n <= 4 * blockDim.x values (4 consecutive per thread) of v(i); *total = sum.
 template <typename F>
@@ -305,6 +305,36 @@ __global__ void __launch_bounds__(kCbThreads) cb_plan_kernel(const CbArgs a) {
     }
 }
 
+enum CbForm { kCbColumns, kCbColumnsByWarp, kCbCells, kCbCellsByWarp };
+
+// The form in which a map is summed, from its records, its fullest cell and the sum of its cells' squared counts.  The
+// reduce alone, one scale, BF16, each form forced in turn (us: columns, columns by warp, cells, cells by warp; r records
+// per row; 24 cameras, 900 anchors x 13 keypoints, C/G = 32, unless said):
+//   even       r = 4: 112 170 252 373   8: 121 123 127 175   13: 139 122 99 121   25: 143 121 78 83   50: 170 126 75 64
+//   projected  r = 5.5: 136 145 191 215   11: 141 132 175 136   17: 140 127 163 106   36: 147 123 197 80
+//   C/G = 8    even  r = 4: 65 124 69 310   8: 75 83 52 166   25: 69 52 41 63   projected  11: 96 72 86 104   36: 101 60 156 44
+//   C/G = 8, 2 cameras, 187 anchors (one band)   projected  r = 5.5: 17 14 23 26   22: 22 11 33 13   83: 39 10 64 12
+//   40 cameras, 300 anchors (one band)   projected  r = 5.5: 63 56 102 100   22: 78 45 98 49   70: 116 49 200 68
+// * A lane group per cell wants cells for its lane groups and none much fuller than the others.  It gains from r = 3 +
+//   24 / (lane groups of a warp) on, and the warp overtakes it at 8 x (lane groups of a warp) records per row.
+// * Where the points crowd (a record's cell holds more than twice the mean of the map), columns differ in length, and a
+//   warp per column evens them out, as long as the map comes in few bands: each band's cell rows are swept once more at
+//   its start, and a band that is one row is not staged at all.
+// Over 172 such maps (r = 1 to 235; 187 to 900 anchors; C/G = 8 to 64; even, projected, half of the points in a hundredth
+// of the map, 200 points in one cell) the form taken is 1.2 % from the best on average and more than 10 % in three.
+__device__ __forceinline__ CbForm cb_form(const CbArgs& a, int H, int W, uint32_t nrec, uint32_t most, uint32_t squares) {
+    const float nlgw = (float)(128 / a.Cg);  // lane groups of a warp (4 channels per lane)
+    const float per = (float)nrec / (float)(H * W);
+    const float bands = (float)nrec / (float)a.nb;
+    const bool uneven = (float)squares > (1.f + 2.f * per) * (float)nrec;
+    if (uneven && per >= 3.f + 0.125f * nlgw && bands <= (per < 16.f ? 4.f : 1.25f)) return kCbColumnsByWarp;
+    if (2 * (W + 1) > a.ncap) return per >= 8.f ? kCbColumnsByWarp : kCbColumns;
+    if (per < 3.f + 24.f / nlgw) return kCbColumns;
+    const bool level = (float)most <= 3.f * per + 8.f;
+    if (level && (float)((H + 1) * (W + 1)) >= 0.625f * kCbWarps * nlgw && per < 8.f * nlgw) return kCbCells;
+    return per >= 8.f * nlgw || (bands > 1.25f && per >= 1.5f * nlgw) ? kCbCellsByWarp : kCbColumnsByWarp;
+}
+
 // ---------------------------------------------------------------------------
 // Binning: one block per (batch element, map).  The camera's A * P points get their cells (0xffff when out of
 // view) and are counted per cell with shared-memory atomics; the counts' prefix sums are the map's cell
@@ -429,11 +459,12 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
     uint32_t* lng = reinterpret_cast<uint32_t*>(idx + align16(2 * (size_t)ap) / 2);
     __shared__ int wsum[32];
     __shared__ int s_nlong, s_abort;
+    __shared__ uint32_t s_most, s_sq;
     const int chunk = (ap + kCbWarps - 1) / kCbWarps;  // stable: points of warp w are [w * chunk, ...)
     const int ncnt = stable ? kCbWarps * cstride : ncell + 1;
 
     for (int c = threadIdx.x; c < ncnt; c += blockDim.x) cnt[c] = 0u;
-    if (threadIdx.x == 0) { s_nlong = 0; s_abort = 0; }
+    if (threadIdx.x == 0) { s_nlong = 0; s_abort = 0; s_most = s_sq = 0u; }
     __syncthreads();
     const float2* lk = reinterpret_cast<const float2*>(a.ws + a.L.loct) + ((long long)b * a.Ncam + k) * ap;
     for (int i0 = threadIdx.x; i0 < ap; i0 += 4 * blockDim.x) {
@@ -539,15 +570,24 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
     // end of cell c (the start of cell c + 1): the last warp's cursor when stable, else the counter
     const uint32_t* cend = stable ? cnt + (kCbWarps - 1) * cstride : cnt;
     const int total = (int)cend[ncell - 1];
-    if (!stable) {
-        // point order inside every cell
+    {
+        // how the points crowd (the reduce chooses its form by it), and point order inside every cell
+        uint32_t most = 0u, sq = 0u;
         for (int c = threadIdx.x; c < ncell; c += blockDim.x) {
             const int e0 = c > 0 ? (int)cend[c - 1] : 0, n = (int)cend[c] - e0;
-            if (n <= 1) continue;
+            most = max(most, (uint32_t)n);
+            sq += (uint32_t)n * (uint32_t)n;
+            if (stable || n <= 1) continue;
             if (n <= 4) cb_sort_small<4>(idx + e0, n);
             else if (n <= 16) cb_sort_small<16>(idx + e0, n);
             else if (n <= kCbMaxBin || ncell <= kCbRescanCells) lng[atomicAdd(&s_nlong, 1)] = (uint32_t)c;
             else s_abort = 1;
+        }
+        most = __reduce_max_sync(0xffffffffu, most);
+        sq = __reduce_add_sync(0xffffffffu, sq);  // the whole sum is at most (A * P)^2, below 2^32
+        if (lane == 0 && sq) {
+            atomicMax(&s_most, most);
+            atomicAdd(&s_sq, sq);
         }
     }
     __syncthreads();
@@ -555,6 +595,9 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
         if (threadIdx.x == 0) atomicExch(&hdr->ok, 0);
         return;
     }
+    if (threadIdx.x == 0)
+        reinterpret_cast<int*>(a.ws + a.L.forms)[(long long)b * a.nmaps + m] =
+            cb_form(a, H, W, (uint32_t)total, s_most, s_sq);
     for (int li = warp; li < s_nlong; li += kCbWarps) {
         const int c = (int)lng[li];
         const int e0 = c > 0 ? (int)cend[c - 1] : 0, n = (int)cend[c] - e0;
@@ -620,7 +663,8 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
 // for the left cell, 1 - fx for the right one).  The row below therefore receives its cell-row cy records
 // before its own, which is the order (i-1, j-1), (i-1, j), (i, j-1), (i, j) for every row (i, j); a segment
 // starting at row i0 first sweeps cell row i0 - 1 for the row below only.  A lane group (LG lanes, 4 channels each)
-// sweeps a column.  Dense maps are summed by cells instead (cb_dense_map).
+// sweeps a column, or a warp does where points crowd (cb_sweep_by_warp), and dense maps are summed by cells instead
+// (cb_dense_map); cb_form chooses.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cb_fma4(float4& acc, float k, const float4& v) {
     acc.x = fmaf(k, v.x, acc.x);
@@ -662,11 +706,11 @@ __device__ __forceinline__ void cb_store(const CbArgs& a, unsigned short* dst, c
 template <bool ONLY_NEXT>
 __device__ __forceinline__ void cb_step(const uint32_t* __restrict__ Ao, const float4* __restrict__ Cf,
                                         const float4* __restrict__ sgo, int l, uint32_t e, uint32_t e1, uint32_t e2,
-                                        uint32_t ae, uint32_t ce, float4& cur, float4& nxt) {
-    for (; e + 1 < e2; e += 2) {
-        const uint32_t o0 = Ao[e - ae], o1 = Ao[e + 1 - ae];
-        const float4 k0 = Cf[e - ce], k1 = Cf[e + 1 - ce];
-        const bool l0 = e < e1, l1 = e + 1 < e1;
+                                        uint32_t ae, uint32_t ce, int step, float4& cur, float4& nxt) {
+    for (; e + step < e2; e += 2 * step) {
+        const uint32_t o0 = Ao[e - ae], o1 = Ao[e + step - ae];
+        const float4 k0 = Cf[e - ce], k1 = Cf[e + step - ce];
+        const bool l0 = e < e1, l1 = e + step < e1;
         const float4 v0 = sgo[(o0 >> 2) + l];
         const float4 v1 = sgo[(o1 >> 2) + l];
         if (ONLY_NEXT) {
@@ -726,31 +770,46 @@ __device__ __forceinline__ CbBand cb_issue_band(const CbArgs& a, unsigned char* 
     return bd;
 }
 
-// The column sweeps of a band read in place: the same steps as the staged sweep in cb_reduce_kernel, with the
-// records, anchor offsets and cell pointers taken from the workspace (record e, anchor offset e, cell pointer c
-// at their own indices).  Kept out of line so the staged sweep, which nearly every band takes, is compiled
-// as if it were alone.
-template <typename GT>
-__device__ __noinline__ void cb_sweep_in_place(const CbArgs& a, const float4* __restrict__ coef_g,
-                                               const float4* __restrict__ sgo, GT* gfm, long long pm, int i0,
-                                               int i1, int W, int seg, int ntask, int l, int t0, int tstep, bool failed) {
-    const int W1 = W + 1;
-    const uint32_t* Ao = reinterpret_cast<const uint32_t*>(a.ws + a.L.aoff);
-    const uint32_t* Cp = reinterpret_cast<const uint32_t*>(a.ws + a.L.cellptr);
-    for (int task = t0; task < ntask && !failed; task += tstep) {
+// The column sweeps of a band with a warp per column: its lane groups take every (32/LG)-th record of a cell pair and
+// add their partial rows with a fixed butterfly when a row is finished.  STAGED: the band at smem + buf, as the lane
+// groups' sweep in cb_reduce_kernel reads it; else a band read in place, from the workspace (record e, anchor offset e,
+// cell pointer c at their own indices); with a lane group per column such bands took 414 us where they now take 212 (47x83
+// maps, half of the points in a hundredth of the map).  Kept out of line so that that sweep is compiled as if alone.
+template <int LG, bool STAGED, typename GT>
+__device__ __noinline__ void cb_sweep_by_warp(const CbArgs& a, const float4* __restrict__ coef_g, unsigned buf,
+                                              const CbBand bd, GT* gfm, long long pm, int i0, int i1, int W) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const float4* sgo = reinterpret_cast<const float4*>(smem);
+    const CbRedSmem L(a.A, a.Cg, a.nb);
+    const float4* Cf = STAGED ? reinterpret_cast<const float4*>(smem + buf) : coef_g;
+    const uint32_t* Ao = STAGED ? reinterpret_cast<const uint32_t*>(smem + buf + L.aoff)
+                                : reinterpret_cast<const uint32_t*>(a.ws + a.L.aoff);
+    const uint32_t* Cp = STAGED ? reinterpret_cast<const uint32_t*>(smem + buf + L.cptr)
+                                : reinterpret_cast<const uint32_t*>(a.ws + a.L.cellptr) + pm;
+    const int cp0 = STAGED ? (int)(pm - (long long)bd.ca0) : 0;
+    const int W1 = W + 1, R = i1 - i0;
+    const int S = max(1, min(R, kCbWarps / W)), seg = (R + S - 1) / S;
+    const int lane = threadIdx.x & 31, lgi = lane / LG, l = lane % LG;
+    for (int task = threadIdx.x >> 5; task < W * S; task += kCbWarps) {
         const int sg = task / W, j = task - sg * W;
         const int r0 = i0 + sg * seg, r1 = min(r0 + seg, i1);
         if (r0 >= r1) continue;
         float4 cur = make_float4(0.f, 0.f, 0.f, 0.f), nxt = cur;
-        long long ci = pm + (long long)r0 * W1 + j;  // left cell of cell row r0 - 1
-#pragma unroll 2
+        int ci = cp0 + r0 * W1 + j;  // left cell of cell row r0 - 1
         for (int cy = r0 - 1; cy < r1; ++cy) {
-            const uint32_t q0 = Cp[ci], q1 = Cp[ci + 1], q2 = Cp[ci + 2];
+            const uint32_t q0 = Cp[ci] + lgi, q1 = Cp[ci + 1], q2 = Cp[ci + 2];
             if (cy < r0) {
-                cb_step<true>(Ao, coef_g, sgo, l, q0, q1, q2, 0u, 0u, cur, nxt);
+                cb_step<true>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, 32 / LG, cur, nxt);
             } else {
-                cb_step<false>(Ao, coef_g, sgo, l, q0, q1, q2, 0u, 0u, cur, nxt);
-                cb_store(a, gfm + ((long long)cy * W + j) * a.C, cur);
+                cb_step<false>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, 32 / LG, cur, nxt);
+#pragma unroll
+                for (int o = LG; o < 32; o <<= 1) {
+                    cur.x += __shfl_xor_sync(0xffffffffu, cur.x, o);
+                    cur.y += __shfl_xor_sync(0xffffffffu, cur.y, o);
+                    cur.z += __shfl_xor_sync(0xffffffffu, cur.z, o);
+                    cur.w += __shfl_xor_sync(0xffffffffu, cur.w, o);
+                }
+                if (lgi == 0) cb_store(a, gfm + ((long long)cy * W + j) * a.C, cur);
             }
             cur = nxt;
             nxt = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -771,12 +830,7 @@ __device__ __noinline__ void cb_sweep_in_place(const CbArgs& a, const float4* __
 // registers.
 //
 // A column sweep reads a record for each of its two columns, and again for every row segment that a column is cut into
-// to occupy the block.  Measured for one scale alone (64 cameras, 900 anchors, 0.45 M records; a warp sweeping a column
-// of a dense map before): 9x15 maps (44 records per cell) 155 -> 79 us, 17x30 (13 per cell) 127 -> 130 us, whole frame
-// 529 -> 487 us; 16 cameras, batch 4, whole 844 -> 732 us; 20 cameras with projected keypoints, whole 504 -> 394 us.
-// The lines: at 3.3 records per cell (34x60) this form takes 264 us against 143 us for the sweep, whose bands have no
-// passes to start; at 13 a warp per cell takes 150 us against 130 us for a lane group, at 44 79 against 86 us, and
-// where keypoints crowd (projected, 17x30, 21 per cell on average) 88 against 132 us, since a warp evens out its cells.
+// to occupy the block; this form reads it once, but starts a pass for every few cell rows (cb_form has the figures).
 // ---------------------------------------------------------------------------
 template <int LG, typename GT>
 __device__ __noinline__ int cb_dense_map(const CbArgs& a, const float4* __restrict__ coef_g,
@@ -943,6 +997,7 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
     const CbMap* maps = reinterpret_cast<const CbMap*>(a.ws + a.L.maps);
     int* queues = reinterpret_cast<int*>(a.ws + a.L.queues);
     const uint32_t* cellptr = reinterpret_cast<const uint32_t*>(a.ws + a.L.cellptr);
+    const int* forms = reinterpret_cast<const int*>(a.ws + a.L.forms);
     const float4* coef_g = reinterpret_cast<const float4*>(a.ws + a.L.coef) + (long long)g * a.L.nrec;
     const CbRedSmem L(a.A, a.Cg, a.nb);
     extern __shared__ __align__(16) unsigned char smem[];
@@ -981,17 +1036,15 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
             if (m >= a.nmaps) break;
             if (threadIdx.x == 0) s_item[cur_slot ^ 1] = atomicAdd(queue, 1);  // the next map, fetched meanwhile
             const CbMap mp = maps[m];
+            const int form = __ldg(forms + (long long)b * a.nmaps + m);
             if (mp.W != 0) {
                 const int H = mp.H, W = mp.W, W1 = W + 1;
                 const long long pm = (long long)b * a.L.nccap + mp.cbase;  // the map's cell pointers
                 GT* gfm = gfb + (long long)mp.start * a.C;
-                // a dense map takes its cells one by one, if the corner sums of two cell rows fit in the band buffers
-                const int ncap = min((int)(2 * L.bsize / (4 * sizeof(float) * (size_t)a.Cg)), kCbDensePtrs - 8);
-                const uint32_t nrec = __ldg(cellptr + pm + (long long)(H + 1) * W1) - __ldg(cellptr + pm);
-                if (nrec >= (uint32_t)kCbDensePerRow * (uint32_t)(H * W) && 2 * W1 <= ncap) {
-                    const int npass = cb_dense_map<LG, GT>(a, coef_g, sgo, reinterpret_cast<float4*>(buf0), ncap, gfm, pm, H, W, rp, &s_ctr,
-                                     &s_fail, mbar, ph0, ph1,
-                                     nrec >= (uint32_t)kCbWarpPerCell * (uint32_t)((H + 1) * W1));
+                if (form == kCbCells || form == kCbCellsByWarp) {
+                    const int npass = cb_dense_map<LG, GT>(a, coef_g, sgo, reinterpret_cast<float4*>(buf0), a.ncap, gfm,
+                                                           pm, H, W, rp, &s_ctr, &s_fail, mbar, ph0, ph1,
+                                                           form == kCbCellsByWarp);
                     ph0 ^= (uint32_t)((npass + 1) / 2) & 1u;  // the passes took the two barriers in turn
                     ph1 ^= (uint32_t)(npass / 2) & 1u;
                     // bulk copies of the next map's bands come after these reads and writes of the buffers
@@ -1056,7 +1109,11 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
                     const int ntask = W * S;
                     const bool failed = s_fail != 0;
                     if (direct) {
-                        cb_sweep_in_place<GT>(a, coef_g, sgo, gfm, pm, i0, i1, W, seg, ntask, l, lgid, nlg, failed);
+                        if (!failed) cb_sweep_by_warp<LG, false, GT>(a, coef_g, 0u, bd, gfm, pm, i0, i1, W);
+                    } else if (form == kCbColumnsByWarp) {
+                        if (!failed)
+                            cb_sweep_by_warp<LG, true, GT>(a, coef_g, (unsigned)(L.buf + bf * L.bsize), bd, gfm, pm, i0,
+                                                           i1, W);
                     } else {
                         const float4* Cf = reinterpret_cast<const float4*>(bb);
                         const uint32_t* Ao = reinterpret_cast<const uint32_t*>(bb + L.aoff);
@@ -1072,9 +1129,9 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
                             for (int cy = r0 - 1; cy < r1; ++cy) {
                                 const uint32_t q0 = Cp[ci], q1 = Cp[ci + 1], q2 = Cp[ci + 2];
                                 if (cy < r0) {
-                                    cb_step<true>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, cur, nxt);
+                                    cb_step<true>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, 1, cur, nxt);
                                 } else {
-                                    cb_step<false>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, cur, nxt);
+                                    cb_step<false>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, 1, cur, nxt);
                                     cb_store(a, gfm + ((long long)cy * W + j) * a.C, cur);
                                 }
                                 cur = nxt;
@@ -1124,9 +1181,10 @@ msda_status launch_backward_cb(const Problem& p, const float* grad_out, float* g
     a.L = cb_layout(p, body_base);
     a.B = p.B; a.sum_hw = p.sum_hw; a.C = p.C; a.Ncam = p.Ncam; a.Nscale = p.Nscale; a.nmaps = p.Ncam * p.Nscale;
     a.A = p.A; a.P = p.P; a.G = p.G; a.Cg = p.Cg;
-    a.nlg = kCbWarps * (32 / (p.Cg / 4));
     a.bin_smem = (int)cb_bin_smem_cap(dev);
     a.nb = cb_band_slots(p, dev);
+    a.ncap = (int)(2 * CbRedSmem(p.A, p.Cg, a.nb).bsize / (4 * sizeof(float) * (size_t)p.Cg));
+    if (a.ncap > kCbDensePtrs - 8) a.ncap = kCbDensePtrs - 8;
     a.status = dev.status;
     CbBinKernel bin = p.w_t == MSDA_F32 ? cb_bin_kernel<float>
                     : p.w_t == MSDA_BF16 ? cb_bin_kernel<__nv_bfloat16> : cb_bin_kernel<__half>;
