@@ -34,9 +34,11 @@ constexpr int kCbWarps = kCbThreads / 32;
 constexpr int kCbMaxMaps = 4096;     // maps the plan's block can sort
 constexpr unsigned short kNoCell = 0xffffu;
 constexpr int kCbMaxBin = 256;       // points of a cell that a warp sorts in registers
-// Cells of a map whose fuller cells are put in order by reading all points again (a larger map with such a cell hands
-// the gradient to the corner-slot path).  A 68x120 map, the finest of the 1080p set, has 8349.
-constexpr int kCbRescanCells = 9472;
+// Fuller cells are put in order by reading the camera's points again, ap / 32 steps of a warp for each, whatever the
+// map's size.  Only where few points lie in a map of many cells is such a call handed to the corner-slot form: that costs
+// 0.25 ms there (320 points in one cell of a 100x100 map, 65 and 315 us), but 0.6 ms with 1200 points, 3.6 ms with 3900
+// and 33 ms with 11700 in one cell (68 and 1.1 ms with a third of 1200 or 3900 in one: 88 and 328, 136 and 755 us).
+constexpr int kCbRescanCells = 9472, kCbRescanPoints = 512;
 constexpr int kCbMaxRows = 1024;     // image rows of a map the reduce's band planner holds
 constexpr int kCbDirect = 1 << 30;   // band-end flag: the band is read in place, not staged
 
@@ -340,12 +342,13 @@ __device__ __forceinline__ CbForm cb_form(const CbArgs& a, int H, int W, uint32_
 // view) and are counted per cell with shared-memory atomics; the counts' prefix sums are the map's cell
 // pointers; the points are placed into their cells (shared-memory atomics again) and every cell's points are
 // sorted by point index (one thread per cell of up to 16 points, a warp per fuller cell, which sorts up to
-// kCbMaxBin points and reads fuller cells off the points again), which makes the
-// order inside a cell the point order whatever the atomics did.  A cell of more than kCbMaxBin points in a map of
-// more than kCbRescanCells cells clears the plan's flag, which hands the whole feature gradient to the corner-slot path.  Then, in record order, each
-// in-view point gets its anchor's offset a * C/G in grad_out's staged copy and, per group g, the weights of its
-// four corners w_g * (x factor * y factor), in the products every other kernel forms.  Blocks past the maps
-// clear the uncovered rows.
+// kCbMaxBin points and reads fuller cells off the points again), which makes the order inside a cell the point
+// order whatever the atomics did.  A cell of more than kCbMaxBin points clears the plan's flag, which hands the
+// whole feature gradient to the corner-slot path, in a map of more than kCbRescanCells cells and at most
+// kCbRescanPoints points.  The counts also give the form in which the reduce sums the map.  Then, in record
+// order, each in-view point gets its anchor's offset a * C/G in grad_out's staged copy and, per group g, the
+// weights of its four corners w_g * (x factor * y factor), in the products every other kernel forms.  Blocks
+// past the maps clear the uncovered rows.
 // ---------------------------------------------------------------------------
 template <int N>
 __device__ __forceinline__ void cb_sort_small(unsigned short* seg, int n) {
@@ -571,6 +574,7 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
     const uint32_t* cend = stable ? cnt + (kCbWarps - 1) * cstride : cnt;
     const int total = (int)cend[ncell - 1];
     {
+        const bool rescan = ncell <= kCbRescanCells || ap > kCbRescanPoints;
         // how the points crowd (the reduce chooses its form by it), and point order inside every cell
         uint32_t most = 0u, sq = 0u;
         for (int c = threadIdx.x; c < ncell; c += blockDim.x) {
@@ -580,7 +584,7 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
             if (stable || n <= 1) continue;
             if (n <= 4) cb_sort_small<4>(idx + e0, n);
             else if (n <= 16) cb_sort_small<16>(idx + e0, n);
-            else if (n <= kCbMaxBin || ncell <= kCbRescanCells) lng[atomicAdd(&s_nlong, 1)] = (uint32_t)c;
+            else if (n <= kCbMaxBin || rescan) lng[atomicAdd(&s_nlong, 1)] = (uint32_t)c;
             else s_abort = 1;
         }
         most = __reduce_max_sync(0xffffffffu, most);
