@@ -19,15 +19,16 @@
 // reproducible.  Nothing is summed over cameras, so a block takes only as
 // many cameras as one list chunk covers (16 of 64 with 13 keypoints and 4
 // scales), in the order of batch element, group, anchor: the blocks that run
-// together read the maps of the same few cameras, and there are enough of them that the last wave is
-// short and that few anchors still fill the GPU.  Alone on the GPU, 64
-// cameras of 1080p maps, 4 warps: 900 anchors 695 -> 397 us, 100 anchors
-// 355 -> 80 us (one block per anchor and all its cameras before); with the
-// weights' lines fetched ahead, as in fwd.cu, inside the step 393 -> 379 us and
-// 540 -> 511 us for 16 cameras of batch 4.  The
-// latency of the corner rows bounds it (3.5 GB from L2, 180 us at the probed
-// gather rate), with three blocks of 8 warps, or six of 4, per SM.  A camera
-// whose locations and sums do not fit in shared memory falls back to the per-point kernel of bwd.cu without its scatter.
+// together read the maps of the same few cameras, and there are enough of
+// them that the last wave is short and that few anchors still fill the GPU.
+// Alone on the GPU, 64 cameras of 1080p maps, 4 warps: 900 anchors 695 -> 397
+// us, 100 anchors 355 -> 80 us (one block per anchor and all its cameras
+// before); with the weights' lines fetched ahead, as in fwd.cu, inside the
+// step 393 -> 379 us and 540 -> 511 us for 16 cameras of batch 4.  The latency
+// of the corner rows bounds it (3.5 GB from L2, 180 us at the probed gather
+// rate), with three blocks of 8 warps, or six of 4, per SM.  A camera whose
+// locations and sums do not fit in shared memory falls back to the per-point
+// kernel of bwd.cu without its scatter.
 #include "common.cuh"
 #include "internal.h"
 #include "units.cuh"
@@ -148,7 +149,7 @@ __global__ void __launch_bounds__(256, NV == 2 ? 3 : (NV == 1 ? 4 : 2)) bwd_locw
     const int chunk = blockDim.x * kUnitsPerThread;
     for (int u0 = 0; u0 < npts; u0 += chunk) {
         const int G = p.G;
-        const int total = build_unit_list(u0, npts, p.P, s_slice.y, p.Nscale, p.Ncam, smap, sbox, sloc, nullptr, ul,
+        const int total = build_unit_list(u0, npts, p.P, s_slice.y, p.Nscale, p.Ncam, smap, sbox, sloc, ul,
                                           [&](int row) {
                                               float* d = gwb + (long long)row * G;
                                               if ((G & 3) == 0) {  // 16-byte aligned rows of G values

@@ -658,9 +658,10 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
 
 // ---------------------------------------------------------------------------
 // Row reduce as column sweeps (grad_feat in FP32, or narrowed once in the features' type: the row's sum is in
-// registers either way, and a caller that wants the narrow gradient saves writing and reading the FP32 one; 16 cameras,
-// batch 4, BF16: a 205 us conversion after a 732 us reduce, against a 734 us reduce alone).  Block j works on channel group g = j % G: it stages grad_out[b, :, group g] in
-// shared memory for b = 0, 1, ... in turn and takes whole maps of (b, g) from that pair's queue.  A map's
+// registers either way, and a caller that wants the narrow gradient saves writing and reading the FP32 one; 16
+// cameras, batch 4, BF16: a 205 us conversion after a 732 us reduce, against a 734 us reduce alone).  Block j
+// works on channel group g = j % G: it stages grad_out[b, :, group g] in shared memory for b = 0, 1, ... in turn
+// and takes whole maps of (b, g) from that pair's queue.  A map's
 // columns, cut into row segments, are swept top to bottom: at cell row cy a column j reads the records of its
 // two cells (cy, j-1) and (cy, j), which are adjacent in record order, and adds each record once to the row it
 // finishes, (cy, j), with weight x * (1 - fy), and once to the row below, (cy+1, j), with weight x * fy (x = fx

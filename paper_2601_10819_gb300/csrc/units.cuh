@@ -3,7 +3,7 @@
 // A block that owns one anchor takes the anchor's point-scales (camera k,
 // keypoint p, scale s), flattened camera-major as u = (k * P + p) * Nscale + s,
 // in chunks of kUnitsPerThread per thread.  Stage A (build_unit_list) culls
-// each point-scale of the chunk (camera box, visibility factor, map range)
+// each point-scale of the chunk (camera box, map range)
 // and locates its bilinear cell once, into a record in shared memory, and
 // lists the in-view ones in increasing u with a block scan.  Stage B (in the
 // kernels) deals the list round-robin to the block's teams, which only load
@@ -25,8 +25,8 @@ struct UnitRec {
     int W;       // map width: rows between y0 and y0 + 1
     float fx, fy;
     int wf;      // (index of the point-scale's weights) << 4 | vx0 | vx1 << 1 | vy0 << 2 | vy1 << 3
-    float scale; // forward kernels: camera factor of the fused occlusion-aware form, else 1; build_unit_list without
-                 // camera factors: the point-scale's number u (the bits of an int)
+    float scale; // forward kernels: camera factor of the fused occlusion-aware form, else 1; build_unit_list: the
+                 // point-scale's number u (the bits of an int)
 };
 
 // Bytes of the record array, its 2-byte list and the scan scratch for `units` entries.
@@ -80,8 +80,8 @@ struct UnitList {
 template <typename Dropped, typename Listed>
 __device__ __forceinline__ int build_unit_list(int u0, int nunits, int P, int Ncam, int Nscale, int pitch,
                                                const MapInfo* __restrict__ smap, const float4* __restrict__ sbox,
-                                               const float2* __restrict__ sloc, const float* __restrict__ svn,
-                                               const UnitList& ul, Dropped dropped, Listed listed) {
+                                               const float2* __restrict__ sloc, const UnitList& ul, Dropped dropped,
+                                               Listed listed) {
     const int per_cam = P * Nscale;
     const int mine = (int)threadIdx.x * kUnitsPerThread;
     unsigned vmask = 0u;
@@ -94,10 +94,9 @@ __device__ __forceinline__ int build_unit_list(int u0, int nunits, int P, int Nc
         const int u = u0 + mine + i;
         if (u < nunits) {
             const float2 uv = sloc[pp * Ncam + k];
-            const float cs = svn ? svn[k] : 1.0f;
             const MapInfo m = smap[k * Nscale + sc];
             Cell c;
-            if (cs != 0.0f && in_box(uv, sbox[k]) && m.W != 0 && locate(uv.x, uv.y, m.H, m.W, c)) {
+            if (in_box(uv, sbox[k]) && m.W != 0 && locate(uv.x, uv.y, m.H, m.W, c)) {
                 UnitRec r;
                 r.row00 = m.start + c.y0 * m.W + c.x0;
                 r.W = m.W;
@@ -105,7 +104,7 @@ __device__ __forceinline__ int build_unit_list(int u0, int nunits, int P, int Nc
                 r.fy = c.fy;
                 r.wf = ((((pp * pitch + k) * Nscale) + sc) << 4) | (c.x0 >= 0 ? 1 : 0) | (c.x0 + 1 < m.W ? 2 : 0) |
                        (c.y0 >= 0 ? 4 : 0) | (c.y0 + 1 < m.H ? 8 : 0);
-                r.scale = svn ? cs : __int_as_float(u);
+                r.scale = __int_as_float(u);
                 ul.rec[mine + i] = r;
                 vmask |= 1u << i;
             } else {
