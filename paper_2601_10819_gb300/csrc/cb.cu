@@ -307,33 +307,42 @@ __global__ void __launch_bounds__(kCbThreads) cb_plan_kernel(const CbArgs a) {
     }
 }
 
-enum CbForm { kCbColumns, kCbColumnsByWarp, kCbCells, kCbCellsByWarp };
+enum CbForm { kCbColumns, kCbColumnsCrowded, kCbColumnsByWarp, kCbCells, kCbCellsByWarp };
 
 // The form in which a map is summed, from its records, its fullest cell and the sum of its cells' squared counts.  The
-// reduce alone, one scale, BF16, each form forced in turn (us: columns, columns by warp, cells, cells by warp; r records
-// per row; 24 cameras, 900 anchors x 13 keypoints, C/G = 32, unless said):
-//   even       r = 4: 112 170 252 373   8: 121 123 127 175   13: 139 122 99 121   25: 143 121 78 83   50: 170 126 75 64
-//   projected  r = 5.5: 136 145 191 215   11: 141 132 175 136   17: 140 127 163 106   36: 147 123 197 80
-//   C/G = 8    even  r = 4: 65 124 69 310   8: 75 83 52 166   25: 69 52 41 63   projected  11: 96 72 86 104   36: 101 60 156 44
-//   C/G = 8, 2 cameras, 187 anchors (one band)   projected  r = 5.5: 17 14 23 26   22: 22 11 33 13   83: 39 10 64 12
-//   40 cameras, 300 anchors (one band)   projected  r = 5.5: 63 56 102 100   22: 78 45 98 49   70: 116 49 200 68
-// * A lane group per cell wants cells for its lane groups and none much fuller than the others.  It gains from r = 3 +
-//   24 / (lane groups of a warp) on, and the warp overtakes it at 8 x (lane groups of a warp) records per row.
-// * Where the points crowd (a record's cell holds more than twice the mean of the map), columns differ in length, and a
-//   warp per column evens them out, as long as the map comes in few bands: each band's cell rows are swept once more at
-//   its start, and a band that is one row is not staged at all.
-// Over 172 such maps (r = 1 to 235; 187 to 900 anchors; C/G = 8 to 64; even, projected, half of the points in a hundredth
-// of the map, 200 points in one cell) the form taken is 1.2 % from the best on average and more than 10 % in three.
+// reduce alone, one scale, BF16, each form forced in turn (us: columns; columns, four records at a time; columns by warp;
+// cells; cells by warp.  r: records per row; 24 cameras, 900 anchors x 13 keypoints, C/G = 32, unless said; crowded:
+// half of the points in a hundredth of the map):
+//   even       r = 4: 109 120 177 253 378    8: 114 123 136 128 179    13: 133 140 128 100 122    25: 143 145 127 78 83
+//              50: 188 166 134 74 62
+//   projected  r = 5.5: 137 136 149 198 220    11: 143 138 139 179 139    17: 146 140 131 175 109
+//              36: 157 143 122 174 79
+//   crowded    r = 1: 239 230 398 240 241    2: 221 212 282 545 637    4: 229 224 256 474 405
+//   C/G = 8    even  r = 4: 64 66 128 68 310    8: 72 75 86 52 166    crowded  r = 2: 129 112 227 143 534
+//              projected  r = 5.5: 106 95 104 108 187    11: 101 89 76 87 103    36: 113 97 63 154 44
+//   C/G = 8, 2 cameras, 187 anchors (one band)   projected  r = 5.5: 18 16 15 23 25    22: 25 20 11 33 12
+//   40 cameras, 300 anchors (one band)   projected  r = 5.5: 64 58 59 105 101    22: 86 74 45 98 48
+// * A lane group per cell wants passes with cells for most lane groups, none much fuller than the others.  It gains from
+//   r = 3 + 28 / (lane groups of a warp) on, and the warp overtakes it at 8 x (lane groups of a warp) records per row.
+// * Where the points crowd (a record's cell holds several times the map's mean), columns differ in length, and a warp
+//   per column evens them out, as long as the map comes in few bands: each band's cell rows are swept once more at its
+//   start, and a band that is one row is not staged at all.
+// Over 354 such maps (r = 0.3 to 235; 187 to 1200 anchors; C/G = 8 to 64) the form taken is 2 % from the best on average;
+// the kernel as a whole takes 0.84 of the time it took with a lane group per column, or a warp from 8 points per row on.
 __device__ __forceinline__ CbForm cb_form(const CbArgs& a, int H, int W, uint32_t nrec, uint32_t most, uint32_t squares) {
     const float nlgw = (float)(128 / a.Cg);  // lane groups of a warp (4 channels per lane)
     const float per = (float)nrec / (float)(H * W);
     const float bands = (float)nrec / (float)a.nb;
     const bool uneven = (float)squares > (1.f + 2.f * per) * (float)nrec;
-    if (uneven && per >= 3.f + 0.125f * nlgw && bands <= (per < 16.f ? 4.f : 1.25f)) return kCbColumnsByWarp;
-    if (2 * (W + 1) > a.ncap) return per >= 8.f ? kCbColumnsByWarp : kCbColumns;
-    if (per < 3.f + 24.f / nlgw) return kCbColumns;
+    if (uneven && per >= (bands > 1.25f ? 7.f : 5.f) && bands <= (per < 16.f ? 4.f : 1.25f)) return kCbColumnsByWarp;
+    if (2 * (W + 1) > a.ncap && per >= 8.f) return kCbColumnsByWarp;
+    if (2 * (W + 1) > a.ncap || per < 3.f + 28.f / nlgw) {
+        const float full = nlgw >= 8.f && per >= 1.5f ? 1.f + 5.f * per : fmaxf(1.f + 12.f * per, 10.f);
+        return nlgw >= 4.f && (float)squares > full * (float)nrec ? kCbColumnsCrowded : kCbColumns;
+    }
     const bool level = (float)most <= 3.f * per + 8.f;
-    if (level && (float)((H + 1) * (W + 1)) >= 0.625f * kCbWarps * nlgw && per < 8.f * nlgw) return kCbCells;
+    const int pass = min(H + 1, a.ncap / (W + 1) - 1) * (W + 1);  // cells of a pass
+    if (level && (float)pass >= 0.625f * kCbWarps * nlgw && per < 8.f * nlgw) return kCbCells;
     return per >= 8.f * nlgw || (bands > 1.25f && per >= 1.5f * nlgw) ? kCbCellsByWarp : kCbColumnsByWarp;
 }
 
@@ -668,7 +677,7 @@ __global__ void __launch_bounds__(kCbThreads, 2) cb_bin_kernel(const CbArgs a) {
 // for the left cell, 1 - fx for the right one).  The row below therefore receives its cell-row cy records
 // before its own, which is the order (i-1, j-1), (i-1, j), (i, j-1), (i, j) for every row (i, j); a segment
 // starting at row i0 first sweeps cell row i0 - 1 for the row below only.  A lane group (LG lanes, 4 channels each)
-// sweeps a column, or a warp does where points crowd (cb_sweep_by_warp), and dense maps are summed by cells instead
+// sweeps a column, or a warp does where points crowd (cb_sweep_crowded), and dense maps are summed by cells instead
 // (cb_dense_map); cb_form chooses.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cb_fma4(float4& acc, float k, const float4& v) {
@@ -707,11 +716,13 @@ __device__ __forceinline__ void cb_store(const CbArgs& a, unsigned short* dst, c
 // One cell row of a column from a staged band: records [e, e2) (record e is coefficient slot e - ce and anchor-offset
 // slot e - ae of the band); records before e1 are the left cell's (corners 1 and 3 reach this column: coefficient .y to
 // the finished row, .w to the row below), the others the right cell's (corners 0 and 2: .x and .z).  ONLY_NEXT: the
-// finished row is not this task's.
-template <bool ONLY_NEXT>
+// finished row is not this task's.  Takes every step-th record, U pairs at a time: one where a pair of cells holds a few
+// records (left to the compiler's unrolling, 7 per row took 237 us, now 211), two where they crowd.
+template <bool ONLY_NEXT, int U>
 __device__ __forceinline__ void cb_step(const uint32_t* __restrict__ Ao, const float4* __restrict__ Cf,
                                         const float4* __restrict__ sgo, int l, uint32_t e, uint32_t e1, uint32_t e2,
                                         uint32_t ae, uint32_t ce, int step, float4& cur, float4& nxt) {
+#pragma unroll U
     for (; e + step < e2; e += 2 * step) {
         const uint32_t o0 = Ao[e - ae], o1 = Ao[e + step - ae];
         const float4 k0 = Cf[e - ce], k1 = Cf[e + step - ce];
@@ -775,15 +786,17 @@ __device__ __forceinline__ CbBand cb_issue_band(const CbArgs& a, unsigned char* 
     return bd;
 }
 
-// The column sweeps of a band with a warp per column: its lane groups take every (32/LG)-th record of a cell pair and
-// add their partial rows with a fixed butterfly when a row is finished.  STAGED: the band at smem + buf, as the lane
-// groups' sweep in cb_reduce_kernel reads it; else a band read in place, from the workspace (record e, anchor offset e,
-// cell pointer c at their own indices); with a lane group per column such bands took 414 us where they now take 212 (47x83
-// maps, half of the points in a hundredth of the map).  Kept out of line so that that sweep is compiled as if alone.
-template <int LG, bool STAGED, typename GT>
-__device__ __noinline__ void cb_sweep_by_warp(const CbArgs& a, const float4* __restrict__ coef_g, unsigned buf,
+// The column sweeps of a band whose points crowd, four records at a time.  BYWARP: a warp per column, its lane groups
+// taking every (32/LG)-th record of a cell pair and adding their partial rows with a fixed butterfly when a row is
+// finished; else a lane group per column.  STAGED: the band at smem + buf, as the sweep in cb_reduce_kernel reads it;
+// else a band read in place, from the workspace (record e, anchor offset e, cell pointer c at their own indices): with
+// a lane group per column such bands took 414 us where a warp takes 212 (47x83 maps, half of the points in a hundredth
+// of the map).  Kept out of line so that the sweep of even maps is compiled as if alone.
+template <int LG, bool BYWARP, bool STAGED, typename GT>
+__device__ __noinline__ void cb_sweep_crowded(const CbArgs& a, const float4* __restrict__ coef_g, unsigned buf,
                                               const CbBand bd, GT* gfm, long long pm, int i0, int i1, int W) {
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int NSLOT = BYWARP ? kCbWarps : kCbThreads / LG, STEP = BYWARP ? 32 / LG : 1;
     const float4* sgo = reinterpret_cast<const float4*>(smem);
     const CbRedSmem L(a.A, a.Cg, a.nb);
     const float4* Cf = STAGED ? reinterpret_cast<const float4*>(smem + buf) : coef_g;
@@ -793,9 +806,9 @@ __device__ __noinline__ void cb_sweep_by_warp(const CbArgs& a, const float4* __r
                                 : reinterpret_cast<const uint32_t*>(a.ws + a.L.cellptr) + pm;
     const int cp0 = STAGED ? (int)(pm - (long long)bd.ca0) : 0;
     const int W1 = W + 1, R = i1 - i0;
-    const int S = max(1, min(R, kCbWarps / W)), seg = (R + S - 1) / S;
-    const int lane = threadIdx.x & 31, lgi = lane / LG, l = lane % LG;
-    for (int task = threadIdx.x >> 5; task < W * S; task += kCbWarps) {
+    const int S = max(1, min(R, NSLOT / W)), seg = (R + S - 1) / S;
+    const int l = (int)threadIdx.x % LG, lgi = BYWARP ? (int)(threadIdx.x & 31) / LG : 0;
+    for (int task = (int)threadIdx.x / (BYWARP ? 32 : LG); task < W * S; task += NSLOT) {
         const int sg = task / W, j = task - sg * W;
         const int r0 = i0 + sg * seg, r1 = min(r0 + seg, i1);
         if (r0 >= r1) continue;
@@ -804,15 +817,17 @@ __device__ __noinline__ void cb_sweep_by_warp(const CbArgs& a, const float4* __r
         for (int cy = r0 - 1; cy < r1; ++cy) {
             const uint32_t q0 = Cp[ci] + lgi, q1 = Cp[ci + 1], q2 = Cp[ci + 2];
             if (cy < r0) {
-                cb_step<true>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, 32 / LG, cur, nxt);
+                cb_step<true, 2>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, STEP, cur, nxt);
             } else {
-                cb_step<false>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, 32 / LG, cur, nxt);
+                cb_step<false, 2>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, STEP, cur, nxt);
+                if constexpr (BYWARP) {
 #pragma unroll
-                for (int o = LG; o < 32; o <<= 1) {
-                    cur.x += __shfl_xor_sync(0xffffffffu, cur.x, o);
-                    cur.y += __shfl_xor_sync(0xffffffffu, cur.y, o);
-                    cur.z += __shfl_xor_sync(0xffffffffu, cur.z, o);
-                    cur.w += __shfl_xor_sync(0xffffffffu, cur.w, o);
+                    for (int o = LG; o < 32; o <<= 1) {
+                        cur.x += __shfl_xor_sync(0xffffffffu, cur.x, o);
+                        cur.y += __shfl_xor_sync(0xffffffffu, cur.y, o);
+                        cur.z += __shfl_xor_sync(0xffffffffu, cur.z, o);
+                        cur.w += __shfl_xor_sync(0xffffffffu, cur.w, o);
+                    }
                 }
                 if (lgi == 0) cb_store(a, gfm + ((long long)cy * W + j) * a.C, cur);
             }
@@ -1106,20 +1121,21 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
                     const int i0 = k ? bend[k - 1] & ~kCbDirect : 0, i1 = bend[k] & ~kCbDirect;
                     const bool direct = (bend[k] & kCbDirect) != 0;
                     const CbBand bd = s_band[bf];
-                    const unsigned char* bb = buf0 + bf * L.bsize;
                     const int R = i1 - i0;
                     int S = nlg / W;
                     S = S < 1 ? 1 : (S > R ? R : S);
                     const int seg = (R + S - 1) / S;
                     const int ntask = W * S;
                     const bool failed = s_fail != 0;
+                    const unsigned buf = (unsigned)(L.buf + bf * L.bsize);
                     if (direct) {
-                        if (!failed) cb_sweep_by_warp<LG, false, GT>(a, coef_g, 0u, bd, gfm, pm, i0, i1, W);
+                        if (!failed) cb_sweep_crowded<LG, true, false, GT>(a, coef_g, 0u, bd, gfm, pm, i0, i1, W);
                     } else if (form == kCbColumnsByWarp) {
-                        if (!failed)
-                            cb_sweep_by_warp<LG, true, GT>(a, coef_g, (unsigned)(L.buf + bf * L.bsize), bd, gfm, pm, i0,
-                                                           i1, W);
+                        if (!failed) cb_sweep_crowded<LG, true, true, GT>(a, coef_g, buf, bd, gfm, pm, i0, i1, W);
+                    } else if (form == kCbColumnsCrowded) {
+                        if (!failed) cb_sweep_crowded<LG, false, true, GT>(a, coef_g, buf, bd, gfm, pm, i0, i1, W);
                     } else {
+                        const unsigned char* bb = smem + buf;
                         const float4* Cf = reinterpret_cast<const float4*>(bb);
                         const uint32_t* Ao = reinterpret_cast<const uint32_t*>(bb + L.aoff);
                         const uint32_t* Cp = reinterpret_cast<const uint32_t*>(bb + L.cptr);
@@ -1134,9 +1150,9 @@ __global__ void __launch_bounds__(kCbThreads, 1) cb_reduce_kernel(const CbArgs a
                             for (int cy = r0 - 1; cy < r1; ++cy) {
                                 const uint32_t q0 = Cp[ci], q1 = Cp[ci + 1], q2 = Cp[ci + 2];
                                 if (cy < r0) {
-                                    cb_step<true>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, 1, cur, nxt);
+                                    cb_step<true, 1>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, 1, cur, nxt);
                                 } else {
-                                    cb_step<false>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, 1, cur, nxt);
+                                    cb_step<false, 1>(Ao, Cf, sgo, l, q0, q1, q2, bd.ea0, bd.e0, 1, cur, nxt);
                                     cb_store(a, gfm + ((long long)cy * W + j) * a.C, cur);
                                 }
                                 cur = nxt;
@@ -1195,13 +1211,13 @@ msda_status launch_backward_cb(const Problem& p, const float* grad_out, float* g
                     : p.w_t == MSDA_BF16 ? cb_bin_kernel<__nv_bfloat16> : cb_bin_kernel<__half>;
     CbRedKernel red = p.gf_t == MSDA_F32 ? cb_red_pick<false>(p.Cg / 4) : cb_red_pick<true>(p.Cg / 4);
     if (!red) return fail(MSDA_ERR_UNSUPPORTED, "msda_backward: no cell-binned reduce for C/G = %d", p.Cg);
+    const long long nbm = (long long)p.B * a.nmaps;
     const size_t bin_smem = (size_t)a.bin_smem;
     const size_t red_smem = CbRedSmem(p.A, p.Cg, a.nb).total;
     if ((st = ensure_smem((const void*)bin, bin_smem, dev)) != MSDA_OK) return st;
     if ((st = ensure_smem((const void*)red, red_smem, dev)) != MSDA_OK) return st;
     const long long tiles = (((long long)p.A * p.P + 31) / 32) * ((p.Ncam + 31) / 32) * p.B;
     cb_plan_kernel<<<(unsigned)(1 + tiles), kCbThreads, 0, stream>>>(a);
-    const long long nbm = (long long)p.B * a.nmaps;
     bin<<<(unsigned)(nbm + 16), kCbThreads, bin_smem, stream>>>(a);
     const int ngb = dev.sm_count / p.G;
     red<<<(unsigned)(ngb * p.G), kCbThreads, red_smem, stream>>>(a);
