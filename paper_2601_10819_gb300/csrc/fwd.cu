@@ -235,12 +235,17 @@ __device__ __forceinline__ void accumulate_anchor_units(const FT* __restrict__ f
         // corner rows, which mostly hit in L2: it starts here, for a whole chunk at once (the weights of a point's scales
         // are consecutive, one line for up to 128 bytes).  64 cameras 278 -> 276 us, 24 cameras fused 144 -> 139 us, 6
         // cameras FP32 59 -> 57 us, 16 cameras batch 4 366 -> 355 us; all of an anchor's weights at the block's start
-        // 281, 139, 56 and 358 us.  Point-scales of 64 bytes and more fill a line by two, and each asks for its own: with
-        // 16 FP32 weights and 2 scales (59 cameras, batch 4) 506 us without any, 514 us with the first one's only, 464 us;
-        // with fewer bytes all of them are no faster (G = 8: 479 and 485 us, 64 cameras 284 and 290 us).
-        for (unsigned v = vmask; v; v &= v - 1) {
-            prefetch_line(wb + (long long)(srec[mine + __ffs(v) - 1].wf >> 4) * G);
-            if (G * sizeof(WT) < 64) break;
+        // 281, 139, 56 and 358 us.  16 FP32 weights fill half a line, and each point-scale asks for its own: 59 cameras,
+        // batch 4, 2 scales 506 us without any, 514 us with the first one's only, 464 us; with fewer weights all of them
+        // are no faster (G = 8: 479 and 485 us).  16-bit weights keep to the first one: 32 of them lose nothing by it (451
+        // us without and with it), and a test of G costs the batched kernel 0.4 %.
+        if constexpr (sizeof(WT) == 4) {
+            for (unsigned v = vmask; v; v &= v - 1) {
+                prefetch_line(wb + (long long)(srec[mine + __ffs(v) - 1].wf >> 4) * G);
+                if (G < 16) break;
+            }
+        } else {
+            if (vmask) prefetch_line(wb + (long long)(srec[mine + __ffs(vmask) - 1].wf >> 4) * G);
         }
         int off = block_excl_scan(__popc(vmask), sscan, sscan + 8);
 #pragma unroll
