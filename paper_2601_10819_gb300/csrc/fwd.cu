@@ -539,9 +539,11 @@ __device__ __forceinline__ uint64_t globaltimer() {
 }
 
 // Three blocks per SM at two vectors per lane, as the single-scene kernel: 16 scenes (762 cameras, 14 161 anchors)
-// 2.93 ms, with the weights' lines fetched ahead 2.82 ms (2.95 ms before both).
+// 2.93 ms, with the weights' lines fetched ahead 2.82 ms (2.95 ms before both).  Four at one vector, and no number at
+// four: asked for one block only, the compiler took 103 registers for 63 and 177 for 144 (6 such scenes of 32 channel
+// groups 1380 us, now 820 us).
 template <typename FT, typename WT, int NV>
-__global__ void __launch_bounds__(256, NV == 2 ? 3 : 1) fwd_batched_kernel(const BatchedArgs p) {
+__global__ void __launch_bounds__(256, NV == 2 ? 3 : (NV == 1 ? 4 : 0)) fwd_batched_kernel(const BatchedArgs p) {
     constexpr int CPL = Elem<FT>::VEC * NV;
     extern __shared__ __align__(16) unsigned char smem[];
     const int tpw = 32 / p.rt;
